@@ -100,8 +100,7 @@ struct lbm_handle {
     int32_t *d_col_fluid = nullptr;
     int16_t *d_wall0 = nullptr;
     LatState *d_st = nullptr;
-    int64_t *d_step = nullptr;
-    unsigned int *d_done = nullptr;
+    int64_t *d_step = nullptr;     // step count, one slot per population buffer
     ColObs *d_cols = nullptr;
     void *d_obs = nullptr;
     // [count][3] A, B and solute totals that the last launch of each
@@ -161,7 +160,7 @@ static void free_all(lbm_handle *h) {
                   h->d_in_off, h->d_masks,
                   h->d_pop[0], h->d_pop[1],
                   h->d_mask, h->d_m, h->d_col_fluid, h->d_wall0, h->d_st,
-                  h->d_step, h->d_done, h->d_cols, h->d_obs, h->d_canon,
+                  h->d_step, h->d_cols, h->d_obs, h->d_canon,
                   h->d_dens, h->d_dep, h->d_maps, h->d_mask_maps, h->d_err,
                   h->d_sched, h->d_sums};
     for (void *p : ps)
@@ -586,8 +585,7 @@ extern "C" lbm_status lbm_create_batch(const lbm_geometry *g,
     AL(h->d_col_fluid, sec);
     AL(h->d_wall0, 2 * sec);
     AL(h->d_st, count);
-    AL(h->d_step, 1);
-    AL(h->d_done, 1);
+    AL(h->d_step, 2);
     AL(h->d_cols, cols);
     if (e == cudaSuccess) e = cudaMalloc(&h->d_obs, count * sizeof(lbm_obs));
     AL(h->d_sums, 3 * count);
@@ -704,9 +702,8 @@ extern "C" lbm_status lbm_create_batch(const lbm_geometry *g,
         bad(cudaMemsetAsync(h->d_pop[0], 0, pop * esz, s2), "memset");
         bad(cudaMemsetAsync(h->d_pop[1], 0, pop * esz, s2), "memset");
         bad(cudaMemsetAsync(h->d_m, 0, node * sizeof(double), s2), "memset");
-        bad(cudaMemsetAsync(h->d_step, 0, sizeof(int64_t), s2), "memset");
+        bad(cudaMemsetAsync(h->d_step, 0, 2 * sizeof(int64_t), s2), "memset");
         bad(cudaMemsetAsync(h->d_err, 0, sizeof(int), s2), "memset");
-        bad(cudaMemsetAsync(h->d_done, 0, sizeof(unsigned), s2), "memset");
     }
     if (st == LBM_OK && h->use_tma) {
         std::string why;
@@ -782,8 +779,8 @@ static StepArgs step_args(lbm_handle *h) {
     a.m = h->d_m;
     a.col_fluid = h->d_col_fluid;
     a.st = h->d_st;
-    a.step = h->d_step;
-    a.done = h->d_done;
+    a.step = h->d_step + h->cur;
+    a.step_next = h->d_step + (h->cur ^ 1);
     a.stall_tx = h->stall_tx;
     a.sums = nullptr;
     return a;
@@ -1080,7 +1077,7 @@ extern "C" lbm_status lbm_save(lbm_handle *h, const char *path) {
     dump(h->d_m, h->node_elems * 8);
     dump(h->d_col_fluid, h->nsec * 4);
     dump(h->d_st, h->count * sizeof(LatState));
-    dump(h->d_step, 8);
+    dump(h->d_step + h->cur, 8);
     ok = (fclose(f) == 0) && ok;
     if (!ok) return fail(h, LBM_EIO, std::string("write failed: ") + path);
     return LBM_OK;
@@ -1204,7 +1201,7 @@ extern "C" lbm_status lbm_autotune(lbm_handle *h, int32_t steps,
         {h->d_m, (size_t)h->node_elems * 8},
         {h->d_col_fluid, (size_t)h->nsec * 4},
         {h->d_st, (size_t)h->count * sizeof(LatState)},
-        {h->d_step, 8}};
+        {h->d_step + cur0, 8}};
     size_t total = 0;
     for (auto &p : parts) total += (p.bytes + 255) / 256 * 256;
     char *snap = nullptr;

@@ -133,8 +133,8 @@ struct StepArgs {
     double *m;
     int32_t *col_fluid;
     LatState *st;
-    int64_t *step;          // completed steps (read at start, bumped at end)
-    unsigned int *done;     // blocks finished in this launch
+    const int64_t *step;    // completed steps, read by every block
+    int64_t *step_next;     // receives *step + 1 (another slot, see next_step)
     // test hook of the bounded waits: bytes that block 0 expects on top of
     // its first tile's copies and that no copy delivers (0 normally)
     int32_t stall_tx;

@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(TX *TY)
     const int ty0 = (local / d.tiles_x) * TY;
     uint8_t *__restrict__ mask = a.mask + d.node_off;
 
-    if (tid == 0) s_t = *(volatile long long *)a.step;
+    if (tid == 0) s_t = *a.step;
     for (int k = tid; k < TL::HY * TL::HX; k += TL::NT) {
         const int hy = k / TL::HX, hx = k - hy * TL::HX;
         const int gy = wrapg(ty0 - 2 + hy, ny), gx = wrapg(tx0 - 2 + hx, nx);
@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(TX *TY)
         tot_add(acc, tot, l, a.sums, tid & 31);
         tot_flush(acc, a.sums, tid & 31);
     }
-    finish_launch(a, t);
+    next_step(a, t);
 }
 
 // ---------------------------------------------------------------------------

@@ -413,7 +413,6 @@ __global__ void __launch_bounds__(TX *TY, (TmaTile<S, TX, TY>::MINB))
     if (tid == 0) {
         for (int j = 0; j < NS; ++j) mbar_init(&bar[j], 1);
         fence_mbar_init();
-        *s_t = *(volatile long long *)a.step;
         bool more = true;
         for (int j = 0; j < NSL; ++j) {
             const TileRec r = more && j < NS ? sched_at(j) : TileRec{-1, 0, 0, 0};
@@ -424,6 +423,7 @@ __global__ void __launch_bounds__(TX *TY, (TmaTile<S, TX, TY>::MINB))
             if (more) issue(r, j, j, j == 0 && blockIdx.x == 0 ? a.stall_tx : 0);
         }
     }
+    if (tid == 32) *s_t = *a.step;  // (beside thread 0's chain of loads)
     __syncthreads();
     const long long t = *s_t;
     const MaskBits mb(t);
@@ -670,7 +670,7 @@ __global__ void __launch_bounds__(TX *TY, (TmaTile<S, TX, TY>::MINB))
         }
     }
     if constexpr (SUM) tot_flush(acc, a.sums, lane);
-    finish_launch(a, t);
+    next_step(a, t);
 }
 
 // ---- host side ---------------------------------------------------------------
