@@ -399,6 +399,44 @@ static size_t plan_tiles(const int32_t *nx, const int32_t *ny, int count,
     return slots;
 }
 
+// The schedule of a handle.  Batches of many tiles per block are dealt in
+// strips (plan_tiles): adjacent tile columns then run at about the same time
+// on different blocks, so their shared halo columns are read from L2.  With
+// few tiles per block the strips (4 tiles at least) are too coarse: 256 x 32
+// at 64 x 8 is 16 tiles on 4 of 152 blocks, and 4096 x 128 leaves some blocks
+// 8 tiles and others 4 where 6.7 is the mean.  There each block takes one
+// run of consecutive tiles in (lattice, tile column, row) order, lists that
+// differ by one tile at most.  Step time, strips / runs: 256 x 32 FP32 16.0 /
+// 6.3 us, 1000 x 60 15.0 / 6.3 us, 4096 x 128 24.6 / 22.7 us (6.7 tiles per
+// block); above that the lost halo sharing costs more than the balance
+// gives: a 1024 x 1024 preform (13.5 tiles) 52.1 / 57.2 us, three 4096 x 128
+// lattices FP16 (20.2 tiles) 51.8 / 53.3 us, so the line is at 8.
+constexpr int kRunTiles = 8;  // most tiles per block dealt as runs
+static size_t deal_tiles(const int32_t *nx, const int32_t *ny, int count,
+                         int tx, int ty, int grid, std::vector<TileRec> &sched) {
+    long long total = 0;
+    for (int l = 0; l < count; ++l)
+        total += (long long)((nx[l] + tx - 1) / tx) * ((ny[l] + ty - 1) / ty);
+    if (total > (long long)kRunTiles * grid)
+        return plan_tiles(nx, ny, count, tx, ty, grid, sched);
+    const size_t slots = (size_t)((total + grid - 1) / grid);
+    sched.assign((size_t)grid * slots, TileRec{-1, 0, 0, 0});
+    // block b: tiles [first, end), end = ceil((b + 1) total / grid)
+    long long t = 0, first = 0, end = (total + grid - 1) / grid;
+    int b = 0;
+    for (int l = 0; l < count; ++l)
+        for (int x = 0; x < nx[l]; x += tx)
+            for (int y = 0; y < ny[l]; y += ty, ++t) {
+                while (t >= end) {
+                    ++b;
+                    first = end;
+                    end = ((b + 1) * total + grid - 1) / grid;
+                }
+                sched[b + (size_t)(t - first) * grid] = TileRec{l, x, y, 0};
+            }
+    return slots;
+}
+
 static bool make_schedule(lbm_handle *h, std::string &why) {
     int grid = 0;
     cudaError_t e = grid_step_tma(h->tx, h->ty, h->store(), &grid);
@@ -412,7 +450,7 @@ static bool make_schedule(lbm_handle *h, std::string &why) {
         ny[l] = h->desc[l].ny;
     }
     std::vector<TileRec> sched;
-    const size_t slots = plan_tiles(nx.data(), ny.data(), h->count, h->tx, h->ty, grid, sched);
+    const size_t slots = deal_tiles(nx.data(), ny.data(), h->count, h->tx, h->ty, grid, sched);
     if (cudaMalloc(&h->d_sched, std::max<size_t>(sched.size(), 1) * sizeof(TileRec)) != cudaSuccess ||
         cudaMemcpy(h->d_sched, sched.data(), sched.size() * sizeof(TileRec),
                    cudaMemcpyHostToDevice) != cudaSuccess) {
