@@ -1,9 +1,10 @@
-// lbm_mlp.cu -- the surrogate network of lbm_mlp.h: forward, backward and
-// Adam kernels.  Every matrix product is one launch of gemm_bf16: BF16
-// operands staged in shared memory, tensor-core mma.sync (m16n8k16, FP32
-// accumulate), and a fused epilogue (bias, tanh, or the tanh derivative of
-// back-propagation).  Operands are read through (row, column) strides, so
-// the transposed products of the backward pass need no transposed copies.
+// lbm_mlp.cu -- the surrogate network of lbm_mlp.h.  A pass over the network
+// is one launch: a block carries 16, 32 or 64 rows of the batch through all
+// layers, forward (k_net<., false>) or forward, loss and back to the first
+// layer (k_net<., true>), with the activations in shared memory.  The weight
+// gradients of all layers are one launch (k_dweight) and so is what follows
+// them (k_finish: the sums over the parts, and Adam).  Products run on the
+// tensor cores with BF16 operands and FP32 accumulation.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -19,214 +20,506 @@
 
 namespace lbmmlp {
 
-constexpr int BM = 64, BN = 64, BK = 32, KP = BK + 8;  // KP: padded row
-constexpr int GEMM_THREADS = 128;                        // 2 x 2 warps
-constexpr int kSplit = 8;  // K split of the weight-gradient products
+constexpr int kMaxLayers = 9;      // L hidden + output
+constexpr int kNetThreads = 256;   // 8 warps side by side along the units
+constexpr int kNetWarps = kNetThreads / 32;
+constexpr int kMaxBlocks = 608;    // most blocks of k_net (4 x 152 SMs)
+constexpr int DT = 64, DR = 64;    // k_dweight: tile side, batch rows a stage
+constexpr int DLD = DT + 8;        // padded row
+constexpr int kDwThreads = 128;    // 2 x 2 warps
 
-enum Epi : int {
-    EPI_PLAIN = 0,      // C = A B
-    EPI_BIAS = 1,       // C = A B + bias[n]
-    EPI_BIAS_TANH = 2,  // C = tanh(A B + bias[n])
-    EPI_DTANH = 3,      // C = (A B) (1 - H[m][n]^2)
+__host__ __device__ constexpr int pad32(int d) { return (d + 31) & ~31; }
+
+// Layer l maps dim[l] inputs to dim[l + 1] units (dim[0] = n_in, the output
+// layer is layer L).  Activations and gradients kept for k_dweight have rows
+// of pad32(dim) BF16 values, zero beyond dim.
+//
+// Weights in BF16 are kept in the order the tensor-core operand wants them:
+// for a tile of 8 units and 32 inputs, lane 4 g + t of a warp owns the 8
+// values of unit g at inputs 2 t, 2 t + 1, 2 t + 8, 2 t + 9 and those 16
+// further, as one 16-byte word, the 32 lanes' words back to back.  wf holds
+// W (the forward products), wt its transpose (the gradients of the
+// activations); both are zero beyond the layer's sizes.
+struct Net {
+    int L;                          // hidden layers
+    int dim[kMaxLayers + 1];
+    long off_w[kMaxLayers], off_b[kMaxLayers];  // in the packed parameters
+    long off_f[kMaxLayers], off_t[kMaxLayers];  // in wf and wt
+    int off_db[kMaxLayers];         // in a block's partial bias gradients
+    int ndb;                        // length of those
+    long np;
+    float *w;
+    __nv_bfloat16 *wf, *wt;
+    float *hs[kMaxLayers];          // FP32 hidden activations, [batch][H]
+    __nv_bfloat16 *act[kMaxLayers]; // inputs of layer l in BF16
+    __nv_bfloat16 *dz[kMaxLayers];  // gradients at layer l's pre-activation
+    float *db;                      // [blocks of k_net][ndb]
+    double *loss;                   // [blocks of k_net]
+    float *parts;                   // [split][np] partial weight gradients
 };
 
-template <class T>
-__device__ __forceinline__ __nv_bfloat16 to_bf16(T v);
-template <>
-__device__ __forceinline__ __nv_bfloat16 to_bf16<float>(float v) {
-    return __float2bfloat16_rn(v);
-}
-template <>
-__device__ __forceinline__ __nv_bfloat16 to_bf16<__nv_bfloat16>(__nv_bfloat16 v) {
-    return v;
+// Place of weight (unit j, input i) of a layer with `in` inputs in wf; the
+// same with the roles swapped in wt.
+__device__ __forceinline__ long frag_at(int j, int i, int in) {
+    const int r = i & 15;
+    return (((long)(j >> 3) * (pad32(in) >> 5) + (i >> 5)) * 32 + (j & 7) * 4 +
+            ((r & 7) >> 1)) * 8 + ((i >> 4) & 1) * 4 + (r >> 3) * 2 + (r & 1);
 }
 
 __device__ __forceinline__ void mma_bf16(float d[4], const unsigned a[4],
-                                         const unsigned b[2]) {
+                                         unsigned b0, unsigned b1) {
     asm volatile(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
         "{%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
         "{%0, %1, %2, %3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldsm4(unsigned r[4], const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+__device__ __forceinline__ void ldsm4t(unsigned r[4], const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+__device__ __forceinline__ void st_bf2(__nv_bfloat16 *p, float a, float b) {
+    *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(a, b);
 }
 
-// C[m][n] (row stride ldc) = epilogue(sum_k A(m, k) B(k, n)), m < M, n < N,
-// with A(m, k) = a[m * sam + k * sak] and B(k, n) = b[k * sbk + n * sbn],
-// both rounded to BF16 on their way into shared memory.  Split K
-// (EPI_PLAIN only): block z sums k in [z kchunk, (z + 1) kchunk) and writes
-// its partial product to c + z * M * ldc (k_sum_parts adds them up).
-template <class TA, class TB>
-__global__ void __launch_bounds__(GEMM_THREADS)
-    gemm_bf16(int M, int N, int K, const TA *__restrict__ a, long sam,
-              long sak, const TB *__restrict__ b, long sbk, long sbn,
-              float *__restrict__ c, long ldc, int epi,
-              const float *__restrict__ bias, const float *__restrict__ h,
-              long ldh, int kchunk) {
-    __shared__ __align__(16) __nv_bfloat16 As[BM][KP];
-    __shared__ __align__(16) __nv_bfloat16 Bs[BN][KP];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int wm = warp >> 1, wn = warp & 1;
-    const int g = lane >> 2, t4 = lane & 3;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
-    float acc[2][4][4] = {};
-    const int kb = blockIdx.z * kchunk;
-    const int ke = min(K, kb + kchunk);
-    c += (long)blockIdx.z * M * ldc;
-    for (int k0 = kb; k0 < ke; k0 += BK) {
-        // A tile, BM x BK: walk the unit-stride index fastest
-        if (sak == 1) {
-#pragma unroll 2
-            for (int j = 0; j < BM * BK / GEMM_THREADS; ++j) {
-                const int e = tid + j * GEMM_THREADS;
-                const int kk = e % BK, mm = e / BK;
-                const int m = m0 + mm, k = k0 + kk;
-                As[mm][kk] = (m < M && k < ke) ? to_bf16(a[m * sam + k]) : zero;
-            }
-        } else {
-#pragma unroll 2
-            for (int j = 0; j < BM * BK / GEMM_THREADS; ++j) {
-                const int e = tid + j * GEMM_THREADS;
-                const int mm = e % BM, kk = e / BM;
-                const int m = m0 + mm, k = k0 + kk;
-                As[mm][kk] = (m < M && k < ke) ? to_bf16(a[m * sam + k * sak]) : zero;
+// One product of a block: its rows (in shared memory, K columns) times a
+// fragment-ordered matrix of N columns, in passes of up to 256 columns; warp
+// v takes `ntw` neighbouring 8-column tiles of a pass.  Every weight is read
+// once per block, from L2 straight into the register that feeds the tensor
+// core: PF words of 32 inputs ahead, and the first PF of the next product
+// before the current one's epilogue.
+template <int MT, int PF>
+struct Product {
+    const uint4 *bp;  // this lane's words of the warp's first tile
+    int kt, cnt;      // words of 32 inputs; tiles of this warp, 0..4
+    int n0;           // first column of the warp
+    uint4 q[PF][4];
+
+    __device__ __forceinline__ void start(const __nv_bfloat16 *wp, int K, int N,
+                                          int pass, int warp, int lane) {
+        kt = pad32(K) >> 5;
+        const int left = min(32, (pad32(N) >> 3) - 32 * pass);
+        const int ntw = (left + kNetWarps - 1) / kNetWarps;
+        const int t0 = 32 * pass + warp * ntw;
+        cnt = max(0, min(ntw, left - warp * ntw));
+        n0 = 8 * t0;
+        bp = reinterpret_cast<const uint4 *>(wp) + (long)t0 * kt * 32 + lane;
+#pragma unroll
+        for (int p = 0; p < PF; ++p) load(p, p);
+    }
+    __device__ __forceinline__ void load(int p, int k) {
+        if (k >= kt) return;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (j < cnt) q[p][j] = __ldg(bp + ((long)j * kt + k) * 32);
+    }
+    __device__ __forceinline__ void run(const __nv_bfloat16 *as, int ld, int lane,
+                                        float acc[MT][4][4]) {
+#pragma unroll
+        for (int mi = 0; mi < MT; ++mi)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[mi][j][e] = 0.f;
+        if (cnt == 0) return;
+        const __nv_bfloat16 *ap = as + (lane & 15) * ld + (lane >> 4) * 8;
+        for (int k0 = 0; k0 < kt; k0 += PF) {
+#pragma unroll
+            for (int p = 0; p < PF; ++p) {
+                if (k0 + p >= kt) break;
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    unsigned af[MT][4];
+#pragma unroll
+                    for (int mi = 0; mi < MT; ++mi)
+                        ldsm4(af[mi], ap + mi * 16 * ld + (k0 + p) * 32 + s * 16);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (j < cnt) {
+                            const unsigned b0 = s ? q[p][j].z : q[p][j].x;
+                            const unsigned b1 = s ? q[p][j].w : q[p][j].y;
+#pragma unroll
+                            for (int mi = 0; mi < MT; ++mi) mma_bf16(acc[mi][j], af[mi], b0, b1);
+                        }
+                }
+                load(p, k0 + p + PF);
             }
         }
-        // B tile, BK x BN, kept n-major: Bs[n][k]
-        if (sbn == 1) {
-#pragma unroll 2
-            for (int j = 0; j < BN * BK / GEMM_THREADS; ++j) {
-                const int e = tid + j * GEMM_THREADS;
-                const int nn = e % BN, kk = e / BN;
-                const int n = n0 + nn, k = k0 + kk;
-                Bs[nn][kk] = (n < N && k < ke) ? to_bf16(b[k * sbk + n]) : zero;
-            }
-        } else {
-#pragma unroll 2
-            for (int j = 0; j < BN * BK / GEMM_THREADS; ++j) {
-                const int e = tid + j * GEMM_THREADS;
-                const int kk = e % BK, nn = e / BK;
-                const int n = n0 + nn, k = k0 + kk;
-                Bs[nn][kk] = (n < N && k < ke) ? to_bf16(b[k * sbk + n * sbn]) : zero;
+    }
+};
+
+// A pass over the network for rows [16 MT blockIdx.x, + 16 MT) and every
+// gridDim.x-th such tile after it.  TRAIN: also the loss, the gradients at
+// every pre-activation (in BF16 for k_dweight) and the block's share of the
+// bias gradients and of the loss; without it y receives the output.
+template <int MT, bool TRAIN>
+__global__ void __launch_bounds__(kNetThreads)
+    k_net(const __grid_constant__ Net net, const float *__restrict__ x,
+          const float *__restrict__ target, int batch, float *__restrict__ y,
+          int ld, float inv_count) {
+    constexpr int BM = 16 * MT;
+    constexpr int PF = MT == 1 ? 6 : MT == 2 ? 4 : 3;
+    extern __shared__ __align__(16) __nv_bfloat16 sm[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int g = lane >> 2, t4 = lane & 3;
+    const int L = net.L;
+    __nv_bfloat16 *cur = sm, *nxt = sm + BM * ld;
+    double lsum = 0.0;
+    Product<MT, PF> pr;
+    float acc[MT][4][4];
+
+    for (int tile = blockIdx.x; tile * BM < batch; tile += gridDim.x) {
+        const int m0 = tile * BM;
+        const bool first = tile == (int)blockIdx.x;
+        pr.start(net.wf + net.off_f[0], net.dim[0], net.dim[1], 0, warp, lane);
+        {  // the inputs, rounded to BF16, zero beyond the batch and n_in
+            const int n_in = net.dim[0], kp = pad32(n_in);
+            for (int e = tid; e < BM * kp; e += kNetThreads) {
+                const int r = e / kp, c = e - r * kp;
+                const bool in = c < n_in && m0 + r < batch;
+                const __nv_bfloat16 v =
+                    __float2bfloat16_rn(in ? x[(long)(m0 + r) * n_in + c] : 0.f);
+                cur[r * ld + c] = v;
+                if (TRAIN && m0 + r < batch) net.act[0][(long)(m0 + r) * kp + c] = v;
             }
         }
         __syncthreads();
+        // ---- forward ------------------------------------------------------
+        for (int l = 0; l <= L; ++l) {
+            const int N = net.dim[l + 1], np32 = pad32(N);
+            const int passes = (np32 + 255) / 256;
+            const float *bias = net.w + net.off_b[l];
+            for (int ps = 0; ps < passes; ++ps) {
+                pr.run(cur, ld, lane, acc);
+                const int n0 = pr.n0, cnt = pr.cnt;
+                if (ps + 1 < passes)
+                    pr.start(net.wf + net.off_f[l], net.dim[l], N, ps + 1, warp, lane);
+                else if (l < L)
+                    pr.start(net.wf + net.off_f[l + 1], N, net.dim[l + 2], 0, warp, lane);
+                else if (TRAIN && L > 0)
+                    pr.start(net.wt + net.off_t[L], N, net.dim[L], 0, warp, lane);
 #pragma unroll
-        for (int kk = 0; kk < BK; kk += 16) {
-            unsigned af[2][4], bfr[4][2];
+                for (int j = 0; j < 4; ++j) {
+                    if (j >= cnt) break;
+                    const int n = n0 + 8 * j + 2 * t4;
+                    const float b0 = n < N ? bias[n] : 0.f;
+                    const float b1 = n + 1 < N ? bias[n + 1] : 0.f;
+                    float d0 = 0.f, d1 = 0.f;  // column sums of the gradient
 #pragma unroll
-            for (int mi = 0; mi < 2; ++mi) {
-                const int r = wm * 32 + mi * 16 + g;
-                af[mi][0] = *reinterpret_cast<const unsigned *>(&As[r][kk + 2 * t4]);
-                af[mi][1] = *reinterpret_cast<const unsigned *>(&As[r + 8][kk + 2 * t4]);
-                af[mi][2] = *reinterpret_cast<const unsigned *>(&As[r][kk + 2 * t4 + 8]);
-                af[mi][3] = *reinterpret_cast<const unsigned *>(&As[r + 8][kk + 2 * t4 + 8]);
+                    for (int mi = 0; mi < MT; ++mi)
+#pragma unroll
+                        for (int hf = 0; hf < 2; ++hf) {
+                            const int r = mi * 16 + hf * 8 + g, m = m0 + r;
+                            float v0 = acc[mi][j][2 * hf] + b0;
+                            float v1 = acc[mi][j][2 * hf + 1] + b1;
+                            if (l < L) {
+                                v0 = n < N ? tanhf(v0) : 0.f;
+                                v1 = n < N ? tanhf(v1) : 0.f;  // N is even here
+                                st_bf2(nxt + r * ld + n, v0, v1);
+                                if (TRAIN && m < batch) {
+                                    st_bf2(net.act[l + 1] + (long)m * np32 + n, v0, v1);
+                                    if (n < N)
+                                        *reinterpret_cast<float2 *>(net.hs[l] + (long)m * N + n) =
+                                            make_float2(v0, v1);
+                                }
+                            } else if (!TRAIN) {
+                                if (m < batch && n < N) y[(long)m * N + n] = v0;
+                                if (m < batch && n + 1 < N) y[(long)m * N + n + 1] = v1;
+                            } else {
+                                // d loss / d y = 2 (y - t) / (rows * outputs), 0
+                                // where the target is unknown (NaN)
+                                float e0 = 0.f, e1 = 0.f;
+                                if (m < batch && n < N) {
+                                    const float tv = target[(long)m * N + n];
+                                    if (!isnan(tv)) e0 = v0 - tv;
+                                }
+                                if (m < batch && n + 1 < N) {
+                                    const float tv = target[(long)m * N + n + 1];
+                                    if (!isnan(tv)) e1 = v1 - tv;
+                                }
+                                lsum += (double)e0 * e0 + (double)e1 * e1;
+                                e0 = 2.0f * e0 * inv_count;
+                                e1 = 2.0f * e1 * inv_count;
+                                d0 += e0;
+                                d1 += e1;
+                                st_bf2(nxt + r * ld + n, e0, e1);
+                                if (m < batch) st_bf2(net.dz[L] + (long)m * np32 + n, e0, e1);
+                            }
+                        }
+                    if (TRAIN && l == L) {
+#pragma unroll
+                        for (int o = 4; o < 32; o <<= 1) {
+                            d0 += __shfl_xor_sync(0xffffffffu, d0, o);
+                            d1 += __shfl_xor_sync(0xffffffffu, d1, o);
+                        }
+                        if (g == 0) {
+                            float *q = net.db + (long)blockIdx.x * net.ndb + net.off_db[l] + n;
+                            if (n < N) q[0] = first ? d0 : q[0] + d0;
+                            if (n + 1 < N) q[1] = first ? d1 : q[1] + d1;
+                        }
+                    }
+                }
             }
+            __syncthreads();
+            __nv_bfloat16 *sw = cur;
+            cur = nxt;
+            nxt = sw;
+        }
+        if constexpr (TRAIN) {
+            // ---- back: the gradient at layer l - 1's pre-activation is
+            // (dz_l W_l) (1 - h^2); a thread meets the h that it wrote
+            for (int l = L; l >= 1; --l) {
+                const int N = net.dim[l], np32 = pad32(N);
+                const int passes = (np32 + 255) / 256;
+                const float *hp = net.hs[l - 1];
+                for (int ps = 0; ps < passes; ++ps) {
+                    pr.run(cur, ld, lane, acc);
+                    const int n0 = pr.n0, cnt = pr.cnt;
+                    if (ps + 1 < passes)
+                        pr.start(net.wt + net.off_t[l], net.dim[l + 1], N, ps + 1, warp, lane);
+                    else if (l > 1)
+                        pr.start(net.wt + net.off_t[l - 1], N, net.dim[l - 1], 0, warp, lane);
 #pragma unroll
-            for (int ni = 0; ni < 4; ++ni) {
-                const int cidx = wn * 32 + ni * 8 + g;
-                bfr[ni][0] = *reinterpret_cast<const unsigned *>(&Bs[cidx][kk + 2 * t4]);
-                bfr[ni][1] = *reinterpret_cast<const unsigned *>(&Bs[cidx][kk + 2 * t4 + 8]);
+                    for (int j = 0; j < 4; ++j) {
+                        if (j >= cnt) break;
+                        const int n = n0 + 8 * j + 2 * t4;
+                        float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+                        for (int mi = 0; mi < MT; ++mi)
+#pragma unroll
+                            for (int hf = 0; hf < 2; ++hf) {
+                                const int r = mi * 16 + hf * 8 + g, m = m0 + r;
+                                float v0 = 0.f, v1 = 0.f;
+                                if (m < batch && n < N) {
+                                    const float2 h = *reinterpret_cast<const float2 *>(
+                                        hp + (long)m * N + n);
+                                    v0 = acc[mi][j][2 * hf] * (1.0f - h.x * h.x);
+                                    v1 = acc[mi][j][2 * hf + 1] * (1.0f - h.y * h.y);
+                                }
+                                d0 += v0;
+                                d1 += v1;
+                                st_bf2(nxt + r * ld + n, v0, v1);
+                                if (m < batch)
+                                    st_bf2(net.dz[l - 1] + (long)m * np32 + n, v0, v1);
+                            }
+#pragma unroll
+                        for (int o = 4; o < 32; o <<= 1) {
+                            d0 += __shfl_xor_sync(0xffffffffu, d0, o);
+                            d1 += __shfl_xor_sync(0xffffffffu, d1, o);
+                        }
+                        if (g == 0 && n < N) {
+                            float *q = net.db + (long)blockIdx.x * net.ndb + net.off_db[l - 1] + n;
+                            q[0] = first ? d0 : q[0] + d0;
+                            q[1] = first ? d1 : q[1] + d1;
+                        }
+                    }
+                }
+                __syncthreads();
+                __nv_bfloat16 *sw = cur;
+                cur = nxt;
+                nxt = sw;
             }
+        }
+    }
+    if constexpr (TRAIN) {
+        __shared__ double sl[kNetWarps];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+        if (lane == 0) sl[warp] = lsum;
+        __syncthreads();
+        if (tid == 0) {
+            double s = 0.0;
+            for (int v = 0; v < kNetWarps; ++v) s += sl[v];
+            net.loss[blockIdx.x] = s;
+        }
+    }
+}
+
+__device__ __forceinline__ void cp16(void *dst, const void *src, bool in) {
+    const int n = in ? 16 : 0;  // 0: the 16 bytes are zeroed
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(n));
+}
+
+// Weight gradients of every layer, dW_l[n][k] = sum over the batch of
+// dz_l[b][n] act_l[b][k]: block x takes a DT x DT tile of one layer, block y
+// `rows` rows of the batch (a multiple of DR), and writes its part to
+// parts[y].  Both operands lie batch-major; ldmatrix transposes them.
+__global__ void __launch_bounds__(kDwThreads)
+    k_dweight(const __grid_constant__ Net net, int batch, int rows) {
+    __shared__ __align__(16) __nv_bfloat16 sa[2][DR][DLD], sb[2][DR][DLD];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int wm = warp >> 1, wn = warp & 1;
+    int l = 0, t = blockIdx.x, kx = 0;
+    for (;; ++l) {
+        kx = (net.dim[l] + DT - 1) / DT;
+        const int n = kx * ((net.dim[l + 1] + DT - 1) / DT);
+        if (t < n) break;
+        t -= n;
+    }
+    const int N = net.dim[l + 1], K = net.dim[l], lda = pad32(N), ldb = pad32(K);
+    const int n0 = t / kx * DT, k0 = t % kx * DT;
+    const int b0 = blockIdx.y * rows, b1 = min(batch, b0 + rows);
+    const __nv_bfloat16 *A = net.dz[l], *B = net.act[l];
+    float acc[2][4][4] = {};
+    auto stage = [&](int s, int r0) {
+#pragma unroll
+        for (int j = 0; j < DR * DT / 8 / kDwThreads; ++j) {
+            const int e = tid + j * kDwThreads, r = e >> 3, c = (e & 7) * 8;
+            const bool row = r0 + r < b1;
+            const bool ia = row && n0 + c < lda, ib = row && k0 + c < ldb;
+            cp16(&sa[s][r][c], ia ? A + (long)(r0 + r) * lda + n0 + c : A, ia);
+            cp16(&sb[s][r][c], ib ? B + (long)(r0 + r) * ldb + k0 + c : B, ib);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    stage(0, b0);
+    for (int r0 = b0, s = 0; r0 < b1; r0 += DR, s ^= 1) {
+        if (r0 + DR < b1) {
+            stage(s ^ 1, r0 + DR);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < DR; kk += 16) {
+            unsigned af[2][4], bf[2][4];
+            const int mr = (lane & 7) + (lane >> 4) * 8, mc = ((lane >> 3) & 1) * 8;
+            const int br = (lane & 7) + ((lane >> 3) & 1) * 8, bc = (lane >> 4) * 8;
+#pragma unroll
+            for (int mi = 0; mi < 2; ++mi)
+                ldsm4t(af[mi], &sa[s][kk + mr][wm * 32 + mi * 16 + mc]);
+#pragma unroll
+            for (int nj = 0; nj < 2; ++nj)
+                ldsm4t(bf[nj], &sb[s][kk + br][wn * 32 + nj * 16 + bc]);
 #pragma unroll
             for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
-                for (int ni = 0; ni < 4; ++ni) mma_bf16(acc[mi][ni], af[mi], bfr[ni]);
+                for (int ni = 0; ni < 4; ++ni)
+                    mma_bf16(acc[mi][ni], af[mi], bf[ni >> 1][(ni & 1) * 2],
+                             bf[ni >> 1][(ni & 1) * 2 + 1]);
         }
         __syncthreads();
     }
+    float *c = net.parts + blockIdx.y * net.np + net.off_w[l];
 #pragma unroll
     for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
         for (int ni = 0; ni < 4; ++ni)
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const int m = m0 + wm * 32 + mi * 16 + g + (q >> 1) * 8;
-                const int n = n0 + wn * 32 + ni * 8 + 2 * t4 + (q & 1);
-                if (m >= M || n >= N) continue;
-                float v = acc[mi][ni][q];
-                if (epi == EPI_BIAS || epi == EPI_BIAS_TANH) v += bias[n];
-                if (epi == EPI_BIAS_TANH) v = tanhf(v);
-                if (epi == EPI_DTANH) {
-                    const float hv = h[m * ldh + n];
-                    v *= 1.0f - hv * hv;
-                }
-                c[m * ldc + n] = v;
+                const int n = n0 + wm * 32 + mi * 16 + (lane >> 2) + (q >> 1) * 8;
+                const int k = k0 + wn * 32 + ni * 8 + 2 * (lane & 3) + (q & 1);
+                if (n < N && k < K) c[(long)n * K + k] = acc[mi][ni][q];
             }
 }
 
-// c[i] = sum over z of parts[z * n + i], in order z = 0, 1, ...
-__global__ void k_sum_parts(const float *__restrict__ parts, int nparts,
-                            long n, float *__restrict__ c) {
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n;
-         i += (long)gridDim.x * blockDim.x) {
-        float v = 0.f;
-        for (int z = 0; z < nparts; ++z) v += parts[z * n + i];
-        c[i] = v;
-    }
+// Layer of parameter i, and whether it is a weight (else a bias).
+__device__ __forceinline__ int layer_of(const Net &net, long i, bool &weight) {
+    int l = net.L;
+    while (l > 0 && i < net.off_w[l]) --l;
+    weight = i < net.off_b[l];
+    return l;
+}
+// The BF16 copies of weight i of layer l.
+__device__ __forceinline__ void put_weight(const Net &net, int l, long i, float v) {
+    const int K = net.dim[l], N = net.dim[l + 1];
+    const int e = (int)(i - net.off_w[l]), j = e / K, k = e - j * K;
+    const __nv_bfloat16 b = __float2bfloat16_rn(v);
+    net.wf[net.off_f[l] + frag_at(j, k, K)] = b;
+    if (l > 0) net.wt[net.off_t[l] + frag_at(k, j, N)] = b;
 }
 
-// dy = 2 (y - t) / (rows * cols) where t is a number, 0 where t is NaN;
-// *loss += sum of (y - t)^2 / (rows * cols) over the numbers.
-__global__ void k_mse(const float *__restrict__ y, const float *__restrict__ t,
-                      long n, float inv_count, float *__restrict__ dy,
-                      double *__restrict__ loss) {
-    __shared__ double sh[256];
-    double s = 0.0;
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n;
-         i += (long)gridDim.x * blockDim.x) {
-        const float tv = t[i];
-        float d = 0.f;
-        if (!isnan(tv)) {
-            d = y[i] - tv;
-            s += (double)d * d;
-        }
-        dy[i] = 2.0f * d * inv_count;
-    }
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) atomicAdd(loss, sh[0] * inv_count);
-}
-
-// db[n] = sum_m dz[m][n] for an M x N row-major matrix.
-__global__ void k_colsum(const float *__restrict__ dz, int M, int N,
-                         float *__restrict__ db) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    float s = 0.f;
-    for (int m = 0; m < M; ++m) s += dz[(long)m * N + n];
-    db[n] = s;
-}
-
-// Adam with bias correction; refreshes the BF16 copy.
-__global__ void k_adam(float *__restrict__ w, __nv_bfloat16 *__restrict__ wb,
-                       const float *__restrict__ gr, float *__restrict__ m1,
-                       float *__restrict__ m2, long n, float lr, float c1,
-                       float c2) {
+// Adam with bias correction on parameter i, and the refreshed BF16 copies.
+struct AdamArgs {
+    float *m1, *m2;
+    float lr, c1, c2;
+};
+__device__ __forceinline__ float adam(const Net &net, const AdamArgs &o, long i, float gv) {
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n;
-         i += (long)gridDim.x * blockDim.x) {
-        const float gv = gr[i];
-        const float a = b1 * m1[i] + (1.0f - b1) * gv;
-        const float v = b2 * m2[i] + (1.0f - b2) * gv * gv;
-        m1[i] = a;
-        m2[i] = v;
-        const float wv = w[i] - lr * (a * c1) / (sqrtf(v * c2) + eps);
-        w[i] = wv;
-        wb[i] = __float2bfloat16_rn(wv);
+    const float a = b1 * o.m1[i] + (1.0f - b1) * gv;
+    const float v = b2 * o.m2[i] + (1.0f - b2) * gv * gv;
+    o.m1[i] = a;
+    o.m2[i] = v;
+    const float wv = net.w[i] - o.lr * (a * o.c1) / (sqrtf(v * o.c2) + eps);
+    net.w[i] = wv;
+    return wv;
+}
+
+// After the parts: sums them, in order, into the gradient (grad, when not
+// null) and, with ADAM, updates the parameters.  Blocks x < nwb take 256
+// parameters each and do the weights among them; the others take 32 bias
+// entries each, 8 threads sharing the k_net blocks' shares of an entry; the
+// last of them also adds up the loss.
+template <bool ADAM>
+__global__ void __launch_bounds__(256)
+    k_finish(const __grid_constant__ Net net, int split, int nblk, int nwb,
+             float *__restrict__ grad, AdamArgs o, float inv_count,
+             double *__restrict__ loss) {
+    const int tid = threadIdx.x;
+    if ((int)blockIdx.x < nwb) {
+        const long i = blockIdx.x * 256L + tid;
+        if (i >= net.np) return;
+        bool weight;
+        const int l = layer_of(net, i, weight);
+        if (!weight) return;
+        float v = 0.f;
+#pragma unroll 8
+        for (int z = 0; z < split; ++z) v += net.parts[z * net.np + i];
+        if (grad) grad[i] = v;
+        if (ADAM) put_weight(net, l, i, adam(net, o, i, v));
+        return;
+    }
+    __shared__ float sv[8][32];
+    __shared__ double sd[256];
+    const int c = (blockIdx.x - nwb) * 32 + (tid & 31), z0 = tid >> 5;
+    float v = 0.f;
+    if (c < net.ndb) {
+#pragma unroll 8
+        for (int z = z0; z < nblk; z += 8) v += net.db[(long)z * net.ndb + c];
+    }
+    sv[z0][tid & 31] = v;
+    __syncthreads();
+    if (z0 == 0 && c < net.ndb) {
+        v = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v += sv[k][tid];
+        int l = 0;
+        while (l < net.L && c >= net.off_db[l + 1]) ++l;
+        const long i = net.off_b[l] + (c - net.off_db[l]);
+        if (grad) grad[i] = v;
+        if (ADAM) adam(net, o, i, v);
+    }
+    if (blockIdx.x == gridDim.x - 1) {
+        double s = 0.0;
+        for (int z = tid; z < nblk; z += 256) s += net.loss[z];
+        sd[tid] = s;
+        __syncthreads();
+        for (int w = 128; w > 0; w >>= 1) {
+            if (tid < w) sd[tid] += sd[tid + w];
+            __syncthreads();
+        }
+        if (tid == 0) *loss = sd[0] * inv_count;
     }
 }
 
-__global__ void k_to_bf16(const float *__restrict__ w,
-                          __nv_bfloat16 *__restrict__ wb, long n) {
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n;
-         i += (long)gridDim.x * blockDim.x)
-        wb[i] = __float2bfloat16_rn(w[i]);
+// The BF16 copies of every weight.
+__global__ void k_pack(const __grid_constant__ Net net) {
+    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < net.np;
+         i += (long)gridDim.x * blockDim.x) {
+        bool weight;
+        const int l = layer_of(net, i, weight);
+        if (weight) put_weight(net, l, i, net.w[i]);
+    }
 }
 
 }  // namespace lbmmlp
@@ -235,14 +528,11 @@ using namespace lbmmlp;
 
 struct lbm_mlp {
     lbm_mlp_shape sh{};
-    long np = 0;
-    std::vector<long> off_w, off_b;  // per layer (L + 1)
-    float *w = nullptr, *grad = nullptr, *m1 = nullptr, *m2 = nullptr;
-    __nv_bfloat16 *wb = nullptr;
-    std::vector<float *> hs;         // hidden activations, [max_batch][H]
-    float *y = nullptr, *dy = nullptr, *dz[2] = {nullptr, nullptr};
-    float *split = nullptr;  // split-K partial products of a weight gradient
+    Net net{};
+    float *m1 = nullptr, *m2 = nullptr;
     double *d_loss = nullptr;
+    int tiles = 0;       // k_dweight tiles of all layers
+    int max_split = 1;   // parts of the weight gradients
     cudaStream_t own = nullptr, stream = nullptr;
     long adam_t = 0;
     std::string err;
@@ -270,88 +560,66 @@ lbm_status fail(lbm_mlp *h, lbm_status st, const std::string &msg) {
                                           cudaGetErrorString(e_));           \
     } while (0)
 
-template <class TA, class TB>
-cudaError_t gemm(cudaStream_t s, int M, int N, int K, const TA *a, long sam,
-                 long sak, const TB *b, long sbk, long sbn, float *c, long ldc,
-                 int epi, const float *bias = nullptr,
-                 const float *hh = nullptr, long ldh = 0) {
-    dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
-    gemm_bf16<TA, TB><<<grid, GEMM_THREADS, 0, s>>>(M, N, K, a, sam, sak, b,
-                                                    sbk, sbn, c, ldc, epi,
-                                                    bias, hh, ldh, K);
+constexpr int kSmemMax = 232448 - 1024;
+
+// Row length of a block's activations in shared memory: 8 values beyond the
+// widest layer, so that the 8 rows an ldmatrix reads lie in different banks.
+int row_len(const lbm_mlp *h) {
+    int d = 0;
+    for (int l = 0; l <= h->net.L + 1; ++l) d = std::max(d, pad32(h->net.dim[l]));
+    return d + 8;
+}
+size_t net_smem(const lbm_mlp *h, int mt) {
+    return (size_t)2 * 16 * mt * row_len(h) * sizeof(__nv_bfloat16);
+}
+
+// 16-row units per block.
+int pick_mt(const lbm_mlp *h, int batch) {
+    const int sms = 152;
+    int mt = batch <= 16 * sms ? 1 : batch <= 32 * sms ? 2 : 4;
+    while (mt > 1 && net_smem(h, mt) > (size_t)kSmemMax) mt >>= 1;
+    return mt;
+}
+
+template <bool TRAIN>
+cudaError_t launch_net(lbm_mlp *h, const float *x, const float *target, int batch,
+                       float *y, float inv_count, int *blocks) {
+    const int mt = pick_mt(h, batch);
+    const int grid = std::min((batch + 16 * mt - 1) / (16 * mt), kMaxBlocks);
+    const size_t sm = net_smem(h, mt);
+    *blocks = grid;
+    const int ld = row_len(h);
+    if (mt == 1)
+        k_net<1, TRAIN><<<grid, kNetThreads, sm, h->stream>>>(h->net, x, target, batch, y, ld, inv_count);
+    else if (mt == 2)
+        k_net<2, TRAIN><<<grid, kNetThreads, sm, h->stream>>>(h->net, x, target, batch, y, ld, inv_count);
+    else
+        k_net<4, TRAIN><<<grid, kNetThreads, sm, h->stream>>>(h->net, x, target, batch, y, ld, inv_count);
     return cudaGetLastError();
 }
 
-// C = A B (M x N, row stride N) with K split over `parts` blocks of
-// columns-of-work when the plain grid is small; the partial products go to
-// `scratch` (parts * M * N floats) and are added in a fixed order.
-template <class TA, class TB>
-cudaError_t gemm_split(cudaStream_t s, int M, int N, int K, const TA *a,
-                       long sam, long sak, const TB *b, long sbk, long sbn,
-                       float *c, float *scratch, int parts) {
-    const int kchunk = ((K + parts - 1) / parts + BK - 1) / BK * BK;
-    parts = (K + kchunk - 1) / kchunk;
-    dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, parts);
-    gemm_bf16<TA, TB><<<grid, GEMM_THREADS, 0, s>>>(M, N, K, a, sam, sak, b,
-                                                    sbk, sbn, scratch, (long)N,
-                                                    EPI_PLAIN, nullptr, nullptr,
-                                                    0, kchunk);
-    cudaError_t e = cudaGetLastError();
+// Gradient of the loss into grad (when not null); adam: also the update.
+cudaError_t train(lbm_mlp *h, const float *x, const float *target, int batch,
+                  float *grad, const AdamArgs *adam) {
+    const float inv = 1.0f / (float)((long)batch * h->sh.n_out);
+    int blocks = 0;
+    cudaError_t e = launch_net<true>(h, x, target, batch, nullptr, inv, &blocks);
     if (e != cudaSuccess) return e;
-    const long n = (long)M * N;
-    k_sum_parts<<<(int)std::min<long>((n + 255) / 256, 1024), 256, 0, s>>>(
-        scratch, parts, n, c);
+    // parts of equal, whole stages of rows
+    const int stages = (batch + DR - 1) / DR;
+    const int per = (stages + h->max_split - 1) / h->max_split;
+    const int split = (stages + per - 1) / per;
+    k_dweight<<<dim3(h->tiles, split), kDwThreads, 0, h->stream>>>(h->net, batch, per * DR);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const int nwb = (int)((h->net.np + 255) / 256), nbb = (h->net.ndb + 31) / 32;
+    if (adam)
+        k_finish<true><<<nwb + nbb, 256, 0, h->stream>>>(h->net, split, blocks, nwb, grad,
+                                                         *adam, inv, h->d_loss);
+    else
+        k_finish<false><<<nwb + nbb, 256, 0, h->stream>>>(h->net, split, blocks, nwb, grad,
+                                                          AdamArgs{}, inv, h->d_loss);
     return cudaGetLastError();
-}
-
-int n_layers_total(const lbm_mlp *h) { return h->sh.n_layers + 1; }
-int in_of(const lbm_mlp *h, int l) { return l == 0 ? h->sh.n_in : h->sh.n_hidden; }
-int out_of(const lbm_mlp *h, int l) {
-    return l == h->sh.n_layers ? h->sh.n_out : h->sh.n_hidden;
-}
-
-// Forward pass into the handle's activations; the output lands in y_out.
-cudaError_t forward(lbm_mlp *h, const float *x, int batch, float *y_out) {
-    const int L = h->sh.n_layers;
-    cudaError_t e = cudaSuccess;
-    for (int l = 0; l <= L && e == cudaSuccess; ++l) {
-        const int K = in_of(h, l), N = out_of(h, l);
-        const float *in = l == 0 ? x : h->hs[l - 1];
-        float *out = l == L ? y_out : h->hs[l];
-        e = gemm(h->stream, batch, N, K, in, (long)K, 1L, h->wb + h->off_w[l],
-                 1L, (long)K, out, (long)N, l == L ? EPI_BIAS : EPI_BIAS_TANH,
-                 h->w + h->off_b[l]);
-    }
-    return e;
-}
-
-// Backward pass from dy (in h->dy) into h->grad.
-cudaError_t backward(lbm_mlp *h, const float *x, int batch) {
-    const int L = h->sh.n_layers, H = h->sh.n_hidden;
-    const float *dzl = h->dy;  // gradient at the pre-activation of layer l
-    int cur = 0;
-    cudaError_t e = cudaSuccess;
-    for (int l = L; l >= 0 && e == cudaSuccess; --l) {
-        const int K = in_of(h, l), N = out_of(h, l);
-        const float *in = l == 0 ? x : h->hs[l - 1];
-        // dW_l[n][k] = sum_b dz[b][n] in[b][k]: a small output and a long
-        // sum over the batch, split into kSplit parts
-        e = gemm_split(h->stream, N, K, batch, dzl, 1L, (long)N, in, (long)K,
-                       1L, h->grad + h->off_w[l], h->split, kSplit);
-        if (e != cudaSuccess) break;
-        k_colsum<<<(N + 127) / 128, 128, 0, h->stream>>>(dzl, batch, N,
-                                                         h->grad + h->off_b[l]);
-        e = cudaGetLastError();
-        if (e != cudaSuccess || l == 0) break;
-        // dz_{l-1}[b][k] = (sum_n dz[b][n] W_l[n][k]) (1 - h_{l-1}[b][k]^2)
-        float *next = h->dz[cur];
-        e = gemm(h->stream, batch, K, N, dzl, (long)N, 1L, h->wb + h->off_w[l],
-                 (long)K, 1L, next, (long)K, EPI_DTANH, nullptr, h->hs[l - 1],
-                 (long)H);
-        dzl = next;
-        cur ^= 1;
-    }
-    return e;
 }
 
 lbm_status check_batch(lbm_mlp *h, int batch) {
@@ -359,16 +627,6 @@ lbm_status check_batch(lbm_mlp *h, int batch) {
     if (h->dead) return LBM_ECUDA;
     if (batch < 1 || batch > h->sh.max_batch)
         return fail(h, LBM_EINVAL, "batch outside 1..max_batch");
-    return LBM_OK;
-}
-
-// loss and dy from the forward output in h->y
-lbm_status loss_and_dy(lbm_mlp *h, const float *target, int batch) {
-    const long n = (long)batch * h->sh.n_out;
-    MCK(h, cudaMemsetAsync(h->d_loss, 0, sizeof(double), h->stream));
-    k_mse<<<(int)std::min<long>((n + 255) / 256, 1024), 256, 0, h->stream>>>(
-        h->y, target, n, 1.0f / (float)n, h->dy, h->d_loss);
-    MCK(h, cudaGetLastError());
     return LBM_OK;
 }
 
@@ -395,43 +653,61 @@ lbm_status lbm_mlp_create(const lbm_mlp_shape *shape, lbm_mlp **out) {
     lbm_mlp *h = new (std::nothrow) lbm_mlp();
     if (!h) return fail(nullptr, LBM_ENOMEM, "host allocation");
     h->sh = s;
-    long np = 0;
+    Net &net = h->net;
+    net.L = s.n_layers;
+    net.dim[0] = s.n_in;
+    for (int l = 1; l <= s.n_layers; ++l) net.dim[l] = s.n_hidden;
+    net.dim[s.n_layers + 1] = s.n_out;
+    long np = 0, nf = 0, nt = 0;
     for (int l = 0; l <= s.n_layers; ++l) {
-        h->off_w.push_back(np);
-        np += (long)out_of(h, l) * in_of(h, l);
-        h->off_b.push_back(np);
-        np += out_of(h, l);
+        const int K = net.dim[l], N = net.dim[l + 1];
+        net.off_w[l] = np;
+        np += (long)N * K;
+        net.off_b[l] = np;
+        np += N;
+        net.off_f[l] = nf;
+        nf += (long)pad32(N) * pad32(K);
+        net.off_t[l] = nt;
+        if (l > 0) nt += (long)pad32(N) * pad32(K);
+        net.off_db[l] = net.ndb;
+        net.ndb += N;
+        h->tiles += ((N + DT - 1) / DT) * ((K + DT - 1) / DT);
     }
-    h->np = np;
+    net.np = np;
+    // parts of a weight gradient: about three blocks per SM
+    h->max_split = std::min(std::max(456 / h->tiles, 1), 16);
     bool ok = true;
     auto al = [&](auto **p, size_t n) {
         if (ok && cudaMalloc(p, std::max<size_t>(n, 1) * sizeof(**p)) != cudaSuccess) ok = false;
     };
-    al(&h->w, np);
-    al(&h->grad, np);
+    al(&net.w, np);
     al(&h->m1, np);
     al(&h->m2, np);
-    al(&h->wb, np);
-    h->hs.assign(s.n_layers, nullptr);
-    for (auto &p : h->hs) al(&p, (size_t)s.max_batch * s.n_hidden);
-    al(&h->y, (size_t)s.max_batch * s.n_out);
-    al(&h->dy, (size_t)s.max_batch * s.n_out);
-    al(&h->dz[0], (size_t)s.max_batch * s.n_hidden);
-    al(&h->dz[1], (size_t)s.max_batch * s.n_hidden);
-    al(&h->d_loss, 1);
-    {
-        long wmax = 0;  // largest weight matrix
-        for (int l = 0; l <= s.n_layers; ++l)
-            wmax = std::max(wmax, (long)out_of(h, l) * in_of(h, l));
-        al(&h->split, (size_t)kSplit * wmax);
+    al(&net.wf, nf);
+    al(&net.wt, nt);
+    for (int l = 0; l <= s.n_layers; ++l) {
+        if (l < s.n_layers) al(&net.hs[l], (size_t)s.max_batch * s.n_hidden);
+        al(&net.act[l], (size_t)s.max_batch * pad32(net.dim[l]));
+        al(&net.dz[l], (size_t)s.max_batch * pad32(net.dim[l + 1]));
     }
+    const size_t blocks = std::min(((size_t)s.max_batch + 15) / 16, (size_t)kMaxBlocks);
+    al(&net.db, blocks * net.ndb);
+    al(&net.loss, blocks);
+    al(&net.parts, (size_t)h->max_split * np);
+    al(&h->d_loss, 1);
     if (ok && cudaStreamCreateWithFlags(&h->own, cudaStreamNonBlocking) != cudaSuccess)
         ok = false;
     h->stream = h->own;
     if (ok) {
-        for (void *p : {(void *)h->w, (void *)h->grad, (void *)h->m1, (void *)h->m2})
+        for (void *p : {(void *)net.w, (void *)h->m1, (void *)h->m2})
             ok = ok && cudaMemset(p, 0, np * sizeof(float)) == cudaSuccess;
-        ok = ok && cudaMemset(h->wb, 0, np * sizeof(__nv_bfloat16)) == cudaSuccess;
+        ok = ok && cudaMemset(net.wf, 0, nf * sizeof(__nv_bfloat16)) == cudaSuccess;
+        ok = ok && cudaMemset(net.wt, 0, nt * sizeof(__nv_bfloat16)) == cudaSuccess;
+        const int a = (int)cudaFuncAttributeMaxDynamicSharedMemorySize;
+        for (const void *f : {(const void *)k_net<1, false>, (const void *)k_net<1, true>,
+                              (const void *)k_net<2, false>, (const void *)k_net<2, true>,
+                              (const void *)k_net<4, false>, (const void *)k_net<4, true>})
+            ok = ok && cudaFuncSetAttribute(f, (cudaFuncAttribute)a, kSmemMax) == cudaSuccess;
     }
     if (!ok) {
         lbm_mlp_destroy(h);
@@ -441,18 +717,17 @@ lbm_status lbm_mlp_create(const lbm_mlp_shape *shape, lbm_mlp **out) {
     return LBM_OK;
 }
 
-int64_t lbm_mlp_param_count(const lbm_mlp *h) { return h ? h->np : -1; }
+int64_t lbm_mlp_param_count(const lbm_mlp *h) { return h ? h->net.np : -1; }
 
 lbm_status lbm_mlp_set_params(lbm_mlp *h, const float *host, int64_t n) {
     if (!h || !host) return LBM_EINVAL;
     if (h->dead) return LBM_ECUDA;
-    if (n != h->np) return fail(h, LBM_EINVAL, "parameter count mismatch");
-    MCK(h, cudaMemcpyAsync(h->w, host, n * sizeof(float), cudaMemcpyHostToDevice,
+    if (n != h->net.np) return fail(h, LBM_EINVAL, "parameter count mismatch");
+    MCK(h, cudaMemcpyAsync(h->net.w, host, n * sizeof(float), cudaMemcpyHostToDevice,
                            h->stream));
     MCK(h, cudaMemsetAsync(h->m1, 0, n * sizeof(float), h->stream));
     MCK(h, cudaMemsetAsync(h->m2, 0, n * sizeof(float), h->stream));
-    k_to_bf16<<<(int)std::min<long>((n + 255) / 256, 4096), 256, 0, h->stream>>>(
-        h->w, h->wb, n);
+    k_pack<<<(int)std::min<long>((n + 255) / 256, 4096), 256, 0, h->stream>>>(h->net);
     MCK(h, cudaGetLastError());
     // the host array may be reused as soon as this returns
     MCK(h, cudaStreamSynchronize(h->stream));
@@ -463,8 +738,8 @@ lbm_status lbm_mlp_set_params(lbm_mlp *h, const float *host, int64_t n) {
 lbm_status lbm_mlp_get_params(lbm_mlp *h, float *host, int64_t n) {
     if (!h || !host) return LBM_EINVAL;
     if (h->dead) return LBM_ECUDA;
-    if (n != h->np) return fail(h, LBM_EINVAL, "parameter count mismatch");
-    MCK(h, cudaMemcpyAsync(host, h->w, n * sizeof(float), cudaMemcpyDeviceToHost,
+    if (n != h->net.np) return fail(h, LBM_EINVAL, "parameter count mismatch");
+    MCK(h, cudaMemcpyAsync(host, h->net.w, n * sizeof(float), cudaMemcpyDeviceToHost,
                            h->stream));
     MCK(h, cudaStreamSynchronize(h->stream));
     return LBM_OK;
@@ -480,7 +755,8 @@ lbm_status lbm_mlp_forward(lbm_mlp *h, const float *x, int32_t batch, float *y) 
     lbm_status st = check_batch(h, batch);
     if (st != LBM_OK) return st;
     if (!x || !y) return fail(h, LBM_EINVAL, "NULL argument");
-    MCK(h, forward(h, x, batch, y));
+    int blocks = 0;
+    MCK(h, launch_net<false>(h, x, nullptr, batch, y, 0.f, &blocks));
     return LBM_OK;
 }
 
@@ -489,11 +765,7 @@ lbm_status lbm_mlp_grad(lbm_mlp *h, const float *x, const float *target,
     lbm_status st = check_batch(h, batch);
     if (st != LBM_OK) return st;
     if (!x || !target || !grad) return fail(h, LBM_EINVAL, "NULL argument");
-    MCK(h, forward(h, x, batch, h->y));
-    if ((st = loss_and_dy(h, target, batch)) != LBM_OK) return st;
-    MCK(h, backward(h, x, batch));
-    MCK(h, cudaMemcpyAsync(grad, h->grad, h->np * sizeof(float),
-                           cudaMemcpyDeviceToDevice, h->stream));
+    MCK(h, train(h, x, target, batch, grad, nullptr));
     return read_loss(h, loss);
 }
 
@@ -503,28 +775,25 @@ lbm_status lbm_mlp_train_step(lbm_mlp *h, const float *x, const float *target,
     if (st != LBM_OK) return st;
     if (!x || !target) return fail(h, LBM_EINVAL, "NULL argument");
     if (!(lr > 0.f)) return fail(h, LBM_EINVAL, "learning rate must be > 0");
-    MCK(h, forward(h, x, batch, h->y));
-    if ((st = loss_and_dy(h, target, batch)) != LBM_OK) return st;
-    MCK(h, backward(h, x, batch));
     ++h->adam_t;
-    const float c1 = (float)(1.0 / (1.0 - std::pow(0.9, (double)h->adam_t)));
-    const float c2 = (float)(1.0 / (1.0 - std::pow(0.999, (double)h->adam_t)));
-    k_adam<<<(int)std::min<long>((h->np + 255) / 256, 4096), 256, 0, h->stream>>>(
-        h->w, h->wb, h->grad, h->m1, h->m2, h->np, lr, c1, c2);
-    MCK(h, cudaGetLastError());
+    const AdamArgs o{h->m1, h->m2, lr,
+                     (float)(1.0 / (1.0 - std::pow(0.9, (double)h->adam_t))),
+                     (float)(1.0 / (1.0 - std::pow(0.999, (double)h->adam_t)))};
+    MCK(h, train(h, x, target, batch, nullptr, &o));
     return read_loss(h, loss);
 }
 
 void lbm_mlp_destroy(lbm_mlp *h) {
     if (!h) return;
     if (h->stream) cudaStreamSynchronize(h->stream);
-    for (void *p : {(void *)h->w, (void *)h->grad, (void *)h->m1, (void *)h->m2,
-                    (void *)h->wb, (void *)h->y, (void *)h->dy,
-                    (void *)h->dz[0], (void *)h->dz[1], (void *)h->d_loss,
-                    (void *)h->split})
+    const Net &net = h->net;
+    for (void *p : {(void *)net.w, (void *)h->m1, (void *)h->m2, (void *)net.wf,
+                    (void *)net.wt, (void *)net.db, (void *)net.loss,
+                    (void *)net.parts, (void *)h->d_loss})
         if (p) cudaFree(p);
-    for (float *p : h->hs)
-        if (p) cudaFree(p);
+    for (int l = 0; l < kMaxLayers; ++l)
+        for (void *p : {(void *)net.hs[l], (void *)net.act[l], (void *)net.dz[l]})
+            if (p) cudaFree(p);
     if (h->own) cudaStreamDestroy(h->own);
     delete h;
 }
