@@ -76,7 +76,7 @@ struct lbm_handle {
     int store() const { return half ? (bf16 ? 2 : 1) : 0; }
     // tile of the step kernel (LBM_TILE overrides, lbm_autotune picks per
     // workload); set by pick_tile
-    int tx = 64, ty = 8;
+    int tx = 64, ty = 4;
     bool use_tma = true;
     std::vector<LatDesc> desc;
     std::vector<int64_t> col_base;   // first column of lattice l (all columns)
@@ -226,13 +226,20 @@ static const void *device_view(const void *p) {
     }
 }
 
-static void pick_tile(lbm_handle *h) {
-    // measured fastest on the batched sweep: 64 x 8 for FP32 storage (one
-    // 512-thread block per SM), 64 x 4 for FP16 (two 256-thread blocks per
-    // SM hide the issue-bound codec better; also fastest on the single
-    // capillary and the preform)
-    h->tx = 64;
-    h->ty = h->half ? 4 : 8;
+static void pick_tile(lbm_handle *h, const lbm_geometry *g) {
+    // 64 x 4, two 256-thread blocks per SM: measured fastest on the batched
+    // sweep and the single capillary in both storages (us per step, 64 x 8 /
+    // 64 x 4: sweep of 40 lattices FP32 267 / 252, FP16 248 / 241; 4096 x 128
+    // FP32 22.4 / 19.8, FP16 21.6 / 19.4).  Where 32 x 4 tiles leave no SM
+    // more than one tile, a step is one tile's latency, which the smaller
+    // block shortens: 256 x 32 (64 tiles) 64 x 4 / 32 x 4: FP32 5.5 / 4.3,
+    // FP16 5.3 / 4.5; beyond (1000 x 60, 480 tiles) 5.6 / 6.6.
+    constexpr int kSms = 152;
+    h->ty = 4;
+    long long small = 0;
+    for (int l = 0; l < h->count; ++l)
+        small += (long long)((g[l].nx + 31) / 32) * ((g[l].ny + 3) / 4);
+    h->tx = small <= kSms ? 32 : 64;
     const char *e = getenv("LBM_TILE");
     if (e) {
         int a = 0, b = 0;
@@ -406,9 +413,9 @@ static size_t plan_tiles(const int32_t *nx, const int32_t *ny, int count,
 // at 64 x 8 is 16 tiles on 4 of 152 blocks, and 4096 x 128 leaves some blocks
 // 8 tiles and others 4 where 6.7 is the mean.  There each block takes one
 // run of consecutive tiles in (lattice, tile column, row) order, lists that
-// differ by one tile at most.  Step time, strips / runs: 256 x 32 FP32 16.0 /
-// 6.3 us, 1000 x 60 15.0 / 6.3 us, 4096 x 128 24.6 / 22.7 us (6.7 tiles per
-// block); above that the lost halo sharing costs more than the balance
+// differ by one tile at most.  Step time at 64 x 8 FP32, strips / runs:
+// 256 x 32 16.0 / 6.3 us, 1000 x 60 15.0 / 6.3 us, 4096 x 128 24.6 / 22.7 us
+// (6.7 tiles per block); above that the lost halo sharing costs more than the balance
 // gives: a 1024 x 1024 preform (13.5 tiles) 52.1 / 57.2 us, three 4096 x 128
 // lattices FP16 (20.2 tiles) 51.8 / 53.3 us, so the line is at 8.
 constexpr int kRunTiles = 8;  // most tiles per block dealt as runs
@@ -541,7 +548,7 @@ extern "C" lbm_status lbm_create_batch(const lbm_geometry *g,
     h->count = count;
     h->half = p[0].precision != LBM_FP32;
     h->bf16 = p[0].precision == LBM_BF16;
-    pick_tile(h);
+    pick_tile(h, g);
 
     // ---- packed ragged layout ------------------------------------------
     h->desc.resize(count);

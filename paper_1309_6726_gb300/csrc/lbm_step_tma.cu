@@ -167,23 +167,31 @@ struct TmaTile {
     static constexpr int DESC_OFF = NS * STAGE;                // NSL x 128
     static constexpr int RHO_OFF = DESC_OFF + NSL * 128;       // 2 frames
     // The tile's post-collision output, [NPL][TY][TX] words, written by
-    // bulk tensor stores (FP32 storage: one output tile where it fits, two
-    // block barriers per tile).  FP16 storage takes one block barrier per
-    // tile (ONE_BAR): tiles of up to 256 nodes store their nodes directly
-    // (coalesced 32-bit stores) and run two blocks per SM (128 registers;
-    // the budget of three, 80 registers, spilled and measured 10 % slower
-    // on the batched sweep at 64 x 4, whose stages leave room for two
-    // blocks only); larger tiles keep two output tiles, so that the store
-    // of one is issued while the next is written.
+    // bulk tensor stores, or (NOUT 0) stored node by node in coalesced
+    // 32-bit stores.  Tiles of up to 256 nodes run two blocks per SM at 128
+    // registers, which hide each other's latencies; they store node by node,
+    // without an output tile, and take one block barrier per tile (ONE_BAR).
+    // For FP32 an output tile of 64 x 4 leaves room for one block only
+    // (sweep of 40 lattices: one 512-thread block of 64 x 8 with an output
+    // tile 267 us per step, two of 64 x 4 with direct stores 252; 4096 x 128:
+    // 22.4 and 19.8).  FP32 32 x 8 fits two blocks with its output tile, and
+    // keeps it: slower on capillaries (308 us on the sweep) but the fastest
+    // where solid nodes are everywhere (1024 x 1024 preform: 44.0 us against
+    // 50.9 without it and 48.4 at 64 x 4).  (FP16: the budget of three
+    // blocks, 80 registers, spilled and measured 10 % slower on the batched
+    // sweep at 64 x 4, whose stages leave room for two blocks only.)  Larger
+    // FP16 tiles keep two output tiles, so that the store of one is issued
+    // while the next is written; FP32 ones one, with two barriers per tile.
     static constexpr int OUT_BYTES = (NPL * NT * 4 + 127) / 128 * 128;
     static constexpr int OUT_OFF = RHO_OFF + 2 * RHO_AL;
-    static constexpr bool ONE_BAR = S::kHalf;
     static constexpr int NOUT =
         S::kHalf ? (NT <= 256 ? 0 : (OUT_OFF + 2 * OUT_BYTES + 128 <= 232448 ? 2 : 0))
-                 : (OUT_OFF + OUT_BYTES + 128 <= 232448 ? 1 : 0);
+        : NT <= 256 ? (TX == 32 && TY == 8 ? 1 : 0)
+                    : (OUT_OFF + OUT_BYTES + 128 <= 232448 ? 1 : 0);
     static constexpr bool TS = NOUT > 0;
+    static constexpr bool ONE_BAR = S::kHalf || !TS;
     // blocks per SM the register budget is set for
-    static constexpr int MINB = S::kHalf && NT <= 256 ? 2 : 1;
+    static constexpr int MINB = NT <= 256 ? 2 : 1;
     static constexpr int BAR_OFF = OUT_OFF + NOUT * OUT_BYTES;
     static constexpr int SMEM = BAR_OFF + 128;
     static_assert(SMEM <= 232448, "shared memory per block");
@@ -533,15 +541,15 @@ __global__ void __launch_bounds__(TX *TY, (TmaTile<S, TX, TY>::MINB))
         }
         // ring of the density frame: the lanes of the first warps take
         // RW consecutive ring cells each (consecutive addresses, no
-        // shared-memory bank conflicts).  FP16 storage: when the previous
-        // tile of this block is the one just above (a strip walks down a
+        // shared-memory bank conflicts).  When the previous tile of this
+        // block is the one just above (a strip walks down a
         // tile column), the top ring row is that tile's last frame row
         // (its last row of nodes and their side ring cells, same step),
         // copied instead of pulled again.
         {
             const TileRec rp = s_rec[(k + NSL - 1) % NSL];
-            const bool above = S::kHalf && k > 0 && rp.lat == rc.lat &&
-                               rp.x0 == tx0 && rp.y0 + TY == ty0;
+            const bool above = k > 0 && rp.lat == rc.lat && rp.x0 == tx0 &&
+                               rp.y0 + TY == ty0;
             const int r = warp * TT::RW + lane;
             if (lane < TT::RW && r < TT::NRING) {
                 int ry, rx;
@@ -553,7 +561,10 @@ __global__ void __launch_bounds__(TX *TY, (TmaTile<S, TX, TY>::MINB))
                 const int rpc = (ry + 1) * TT::BX + rx - 1 + TT::XO;
                 float2 q = make_float2(0.f, 0.f);
                 if (above && ry == 0) {
-                    q = reinterpret_cast<const float2 *>(srho((k + 1) & 1))[TY * TT::RX + rx];
+                    const float *fp = srho((k + 1) & 1);
+                    const int pf = TY * TT::RX + rx;
+                    q = S::kHalf ? reinterpret_cast<const float2 *>(fp)[pf]
+                                 : make_float2(fp[pf], fp[TT::RX * TT::RY + pf]);
                 } else if (!(sm[rmc] & mb.force)) {
                     // per lane: a warp-uniform choice here measured slower
                     const unsigned rbb = nb_bits<TT, -1>(sm, rmc, mb.pull);
