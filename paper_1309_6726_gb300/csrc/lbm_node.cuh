@@ -117,6 +117,23 @@ __device__ __forceinline__ void store_node22(const StepArgs &a,
                 fA, fB, g);
 }
 
+// The same for a node's periodic images in the ghost band.
+__device__ __forceinline__ void store_ghosts22(const StepArgs &a,
+                                               const LatDesc &d, int x, int y,
+                                               int own, const float fA[Q],
+                                               const float fB[Q],
+                                               const float g[QS]) {
+    for_ghosts(x, y, d.nx, d.ny, d.pitch, own,
+               [&](int off) { store_node22(a, d, off, fA, fB, g); });
+}
+__device__ __forceinline__ void store_ghosts16(const StepArgs &a,
+                                               const LatDesc &d, int x, int y,
+                                               int own, const uint32_t v[NW16]) {
+    uint32_t *out = static_cast<uint32_t *>(a.fout) + d.pop_off;
+    for_ghosts(x, y, d.nx, d.ny, d.pitch, own,
+               [&](int off) { store_words16(out + off, (int)d.plane, v); });
+}
+
 // Martys-Chen cohesion and adhesion forces and the Shan-Chen velocity
 // shift of a fluid node (readings c1, c3, c4):
 //   F_s = rho_s (G_ads,s sum_i w_i s(x + e_i) e_i
@@ -168,9 +185,8 @@ __device__ __forceinline__ Shift forces_shift(const LatDesc &d, float rA,
 //   fA, fB, g: post-streaming populations of the node (g pulled already);
 //   rhoA_nb / rhoB_nb: densities at x + e_i (index 1..8; 0 if solid in s_t);
 //   snb: bit i set if x + e_i is solid in s_t;  ns: solid D2Q4 links.
-// put(fA, fB, g) writes the node's own post-collision values; its periodic
-// images in the ghost band are written here.  want: also sets tot to the
-// node's fluid content (NodeTot).
+// put(fA, fB, g) writes the node's post-collision values wherever they are
+// kept.  want: also sets tot to the node's fluid content (NodeTot).
 // Returns true if the node reached the threshold in this step.
 template <class Put>
 __device__ __forceinline__ bool fluid_update(
@@ -232,9 +248,6 @@ __device__ __forceinline__ bool fluid_update(
         tot.c = (g[0] + g[2]) + (g[1] + g[3]);
     }
     put(fA, fB, g);
-    // periodic images in the ghost band
-    for_ghosts(gx, gy, d.nx, d.ny, d.pitch, own,
-               [&](int off) { store_node22(a, d, off, fA, fB, g); });
     return flagged;
 }
 
@@ -316,7 +329,7 @@ __device__ __forceinline__ float2 rcp2_guard(float2 x, float lim) {
 //   snb, ns: as for fluid_update.
 // The forces and the shift are those of forces_shift (readings c1, c3, c4),
 // formed for both components at once.  put(words) writes the node's 15
-// stored words; its periodic images in the ghost band are written here.
+// stored words wherever they are kept.
 // want: also sets tot to the node's fluid content (NodeTot).
 // Returns true if the node reached the threshold in this step.
 template <class F, class Put>
@@ -396,10 +409,6 @@ __device__ __forceinline__ bool fluid_update16(
         tot.c = 0.25f * ((g[0] + g[2]) + (g[1] + g[3]));
     }
     put(v);
-    // periodic images in the ghost band
-    uint32_t *out = static_cast<uint32_t *>(a.fout) + d.pop_off;
-    for_ghosts(gx, gy, d.nx, d.ny, d.pitch, own,
-               [&](int off) { store_words16(out + off, (int)d.plane, v); });
     return flagged;
 }
 

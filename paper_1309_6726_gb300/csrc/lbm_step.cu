@@ -283,6 +283,7 @@ __global__ void __launch_bounds__(TX *TY)
                     [&](const uint32_t *v) {
                         store_words16(static_cast<uint32_t *>(a.fout) + d.pop_off + own,
                                       (int)d.plane, v);
+                        store_ghosts16(a, d, gx, gy, own, v);
                     },
                     want, tot);
             } else {
@@ -290,6 +291,7 @@ __global__ void __launch_bounds__(TX *TY)
                     a, d, l, t, gx, gy, own, fA, fB, g, rAn, rBn, snb, ns,
                     [&](const float *pa, const float *pb, const float *pg) {
                         store_node22(a, d, own, pa, pb, pg);
+                        store_ghosts22(a, d, gx, gy, own, pa, pb, pg);
                     },
                     want, tot);
             }
