@@ -27,6 +27,12 @@ cudaError_t launch_step_tma(const StepArgs &a, const CUtensorMap *pop_maps,
                             int nslots, int grid, int tx, int ty, int store,
                             int *err, cudaStream_t s);
 cudaError_t grid_step_tma(int tx, int ty, int store, int *grid);
+bool plan_cluster(const int32_t *nx, const int32_t *ny, int count, int *tx,
+                  int *ty, int *csize);
+int active_clusters(int tx, int ty, int store, int csize);
+cudaError_t launch_step_cluster(const StepArgs &a, int count, int nsteps,
+                                int tx, int ty, int csize, int store,
+                                cudaStream_t s);
 int tma_box_x(int tx);
 int tma_mask_box_x(int tx);
 __global__ void k_unstream(const LatDesc *, int, const float *,
@@ -78,6 +84,9 @@ struct lbm_handle {
     // workload); set by pick_tile
     int tx = 64, ty = 4;
     bool use_tma = true;
+    // small lattices advance several steps per launch, one thread block
+    // cluster of csize tiles of ctx by cty nodes each (0: they do not)
+    int csize = 0, ctx = 0, cty = 0;
     std::vector<LatDesc> desc;
     std::vector<int64_t> col_base;   // first column of lattice l (all columns)
     std::vector<int64_t> in_off_host;  // first node of lattice l, unpadded (count + 1)
@@ -250,6 +259,21 @@ static void pick_tile(lbm_handle *h, const lbm_geometry *g) {
     }
     const char *k = getenv("LBM_KERNEL");
     if (k && strcmp(k, "direct") == 0) h->use_tma = false;
+    // The clusters of all lattices have to fit the device at once, so that
+    // the handle advances at one tile's latency per step (figures at
+    // k_step_cluster).  (A tile or kernel asked for by name is used for every
+    // step.)
+    if (!e && h->use_tma) {
+        std::vector<int32_t> nx(h->count), ny(h->count);
+        for (int l = 0; l < h->count; ++l) {
+            nx[l] = g[l].nx;
+            ny[l] = g[l].ny;
+        }
+        int c = 0;
+        if (plan_cluster(nx.data(), ny.data(), h->count, &h->ctx, &h->cty, &c) &&
+            active_clusters(h->ctx, h->cty, h->store(), c) >= h->count)
+            h->csize = c;
+    }
     const char *gr = getenv("LBM_GRAPH");
     if (gr && strcmp(gr, "0") == 0) h->use_graph = false;
     // test hook of the failure path: the first step's first tile of block 0
@@ -854,6 +878,9 @@ static cudaError_t launch_one(lbm_handle *h, bool sum) {
 // Steps per captured graph: even, so a replay starts and ends with the
 // same population buffer as input.
 static const int kGraphSteps = 16;
+// Steps per cluster launch at most (a launch stays around a millisecond), and
+// the shortest call that uses them: a launch also loads and stores the state.
+static const int kClusterSteps = 512, kClusterMin = 4;
 
 // Captures kGraphSteps launches starting from buffer 0 into h->graph[sum];
 // sum: the last one adds up the lattice totals.
@@ -883,6 +910,25 @@ extern "C" lbm_status lbm_step(lbm_handle *h, int64_t n) {
     // The last launch of the call adds up the lattice totals of the state it
     // leaves (a replay that ends the call uses the graph whose last launch
     // sums).
+    // Lattices that fit a cluster: all but the last step on chip, up to
+    // kClusterSteps per launch.  (Not while the caller captures the stream:
+    // a launch moves the state to the other buffer whatever its step count,
+    // and a graph replayed from one buffer counts on one move per step.)
+    if (h->csize > 0 && h->stall_tx == 0 && n >= kClusterMin) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess) {
+            cudaGetLastError();
+            cap = cudaStreamCaptureStatusActive;
+        }
+        while (cap == cudaStreamCaptureStatusNone && n > 1) {
+            const int m = (int)std::min<int64_t>(n - 1, kClusterSteps);
+            CK(h, launch_step_cluster(step_args(h), h->count, m, h->ctx, h->cty,
+                                      h->csize, h->store(), h->stream));
+            h->cur ^= 1;
+            h->steps += m;
+            n -= m;
+        }
+    }
     // Whole groups of kGraphSteps steps replay one captured graph (the
     // step count lives on the device, so the graph needs no new arguments)
     // (a pending test stall is never captured into the graph)
@@ -1272,6 +1318,9 @@ extern "C" lbm_status lbm_autotune(lbm_handle *h, int32_t steps,
                           {false, 32, 8}, {false, 32, 4}, {false, 64, 4},
                           {false, 128, 4}};
     const Cand orig = {h->use_tma, h->tx, h->ty};
+    // the variants are what a single step uses; steps on chip are set aside
+    const int csize0 = h->csize;
+    h->csize = 0;
     Cand best = orig;
     double best_ms = 1e300;
     lbm_status st = LBM_OK;
@@ -1305,6 +1354,7 @@ extern "C" lbm_status lbm_autotune(lbm_handle *h, int32_t steps,
         h->steps = steps0;
         h->sums_step = -1;
     }
+    h->csize = csize0;
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     cudaFree(snap);
