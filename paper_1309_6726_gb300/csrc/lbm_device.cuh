@@ -268,6 +268,9 @@ struct F16 {
         const __half2 h = __floats2half2_rn(a, b);
         return *reinterpret_cast<const uint32_t *>(&h);
     }
+    static __device__ __forceinline__ float2 unpack(uint32_t w) {
+        return __half22float2(*reinterpret_cast<const __half2 *>(&w));
+    }
     static __device__ __forceinline__ float fma(uint16_t h, uint16_t s, float c) {
         float r;
         asm("fma.rn.f32.f16 %0, %1, %2, %3;" : "=f"(r) : "h"(h), "h"(s), "f"(c));
@@ -281,6 +284,9 @@ struct BF16 {
     static __device__ __forceinline__ uint32_t pack(float a, float b) {
         const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
         return *reinterpret_cast<const uint32_t *>(&h);
+    }
+    static __device__ __forceinline__ float2 unpack(uint32_t w) {
+        return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w));
     }
     static __device__ __forceinline__ float fma(uint16_t h, uint16_t s, float c) {
         float r;
@@ -337,14 +343,27 @@ __device__ __forceinline__ float2 enc_ab(const float2 f[Q], uint32_t w[8],
     const bool ub = f[0].y >= f[0].x ? va.y <= f[0].y : wall && va.y <= 4.f * f[0].y;
     wv[0] = F::pack(ua ? vx.x : 0.f, ub ? vx.y : 0.f);
     wv[1] = F::pack(ua ? vy.x : 0.f, ub ? vy.y : 0.f);
+    // -2^10 r_i for every direction (a power of two commutes with every
+    // rounding here), both components at once; the diagonals continue from
+    // the axis they share their x term with, as ref_dir forms them
+    const float2 s0 = mul2(f2s(-kDevScale), f[0]);
+    const float2 ux = mul2(f2s(-kDevScale), F::unpack(wv[0]));
+    const float2 uy = mul2(f2s(-kDevScale), F::unpack(wv[1]));
+    float2 r[Q];
+    r[1] = add2(s0, ux);
+    r[3] = sub2(s0, ux);
+    r[2] = add2(s0, uy);
+    r[4] = sub2(s0, uy);
+    r[5] = add2(r[1], uy);
+    r[8] = sub2(r[1], uy);
+    r[6] = add2(r[3], uy);
+    r[7] = sub2(r[3], uy);
     float2 e = f2s(0.f);
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
-        const float2 r = make_float2(ref_dir<F>(i, false, f[0].x, lo16(wv[0]), lo16(wv[1])),
-                                     ref_dir<F>(i, false, f[0].y, hi16(wv[0]), hi16(wv[1])));
         // f^_i - r_i is exact where the two are within a factor of two
         // (everywhere the deviation is small), the scale exact
-        const float2 dv = mul2(sub2(f[i], r), f2s(kDevScale));
+        const float2 dv = fma2(f[i], f2s(kDevScale), r[i]);
         const uint32_t h = F::pack(dv.x, dv.y);
         // the quantisation errors dv - round(dv), exact
         const float2 q = make_float2(F::fma(lo16(h), F::kMinusOne, dv.x),

@@ -340,11 +340,11 @@ __device__ __forceinline__ bool fluid_update16(
     float2 jx, jy;
     mom2(f, jx, jy);
     // ---- Martys-Chen forces: A feels B, B feels A -------------------------
-    float2 sw[Q];
-#pragma unroll
-    for (int i = 1; i < Q; ++i) sw[i] = make_float2(nb[i].y, nb[i].x);
+    // (the stencil on the pairs as they are, its two sums swapped)
     float2 cx2, cy2;
-    stencil2(sw, cx2, cy2);
+    stencil2(nb, cx2, cy2);
+    cx2 = make_float2(cx2.y, cx2.x);
+    cy2 = make_float2(cy2.y, cy2.x);
     float adx = 0.f, ady = 0.f;
     if (snb != 0u) {  // solid neighbours: adhesion stencil
         float sv[Q];
