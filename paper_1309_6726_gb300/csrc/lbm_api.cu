@@ -96,13 +96,14 @@ struct lbm_handle {
     int64_t pop_elems = 0, node_elems = 0;  // 32-bit words, mask bytes
     size_t max_nodes = 0;            // largest nx*ny
     // device
+    void *d_arena = nullptr;       // what follows, but for what is said to be apart
     LatDesc *d_desc = nullptr;
-    int32_t *d_tile_lat = nullptr;
+    int32_t *d_tile_lat = nullptr; // direct kernel's tiles (apart)
     int32_t *d_col_lat = nullptr;
     int64_t *d_col_base = nullptr;
     int64_t *d_in_off = nullptr;       // node then row prefixes, 2 (count + 1)
     int64_t total_rows = 0;
-    uint8_t *d_masks = nullptr;        // all solid masks, unpadded (on first use)
+    uint8_t *d_masks = nullptr;        // all solid masks, unpadded (apart, on first use)
     void *d_pop[2] = {nullptr, nullptr};
     uint8_t *d_mask = nullptr;
     double *d_m = nullptr;
@@ -124,7 +125,7 @@ struct lbm_handle {
     // output stores
     CUtensorMap *d_maps = nullptr;
     CUtensorMap *d_mask_maps = nullptr; // [count] mask maps
-    TileRec *d_sched = nullptr;        // TMA kernel: tiles of each block
+    TileRec *d_sched = nullptr;        // TMA kernel: tiles of each block (apart)
     int sched_grid = 0, sched_slots = 0;
     // kGraphSteps steps from cur == 0; [1]: the last launch sums the
     // lattice totals (the replay that ends an lbm_step call)
@@ -164,14 +165,31 @@ static cudaError_t dalloc(T **p, size_t n) {
     return cudaMalloc((void **)p, std::max<size_t>(n, 1) * sizeof(T));
 }
 
+// Buffers of one device allocation: each is registered with its size, then
+// all are placed, 256 bytes apart at least.  (One allocation per buffer and
+// its release were 0.25 of the 0.41 ms that creating and destroying a 131 x 13
+// lattice took.)
+struct Arena {
+    struct Item { void **p; size_t at; };
+    std::vector<Item> items;
+    size_t bytes = 0;
+    template <class T>
+    size_t add(T **p, size_t n) {
+        const size_t at = bytes;
+        items.push_back({(void **)p, at});
+        bytes += (std::max<size_t>(n, 1) * sizeof(T) + 255) / 256 * 256;
+        return at;
+    }
+    cudaError_t place(void **base) {
+        cudaError_t e = cudaMalloc(base, std::max<size_t>(bytes, 256));
+        if (e == cudaSuccess)
+            for (Item &i : items) *i.p = (char *)*base + i.at;
+        return e;
+    }
+};
+
 static void free_all(lbm_handle *h) {
-    void *ps[] = {h->d_desc, h->d_tile_lat, h->d_col_lat, h->d_col_base,
-                  h->d_in_off, h->d_masks,
-                  h->d_pop[0], h->d_pop[1],
-                  h->d_mask, h->d_m, h->d_col_fluid, h->d_wall0, h->d_st,
-                  h->d_step, h->d_cols, h->d_obs, h->d_canon,
-                  h->d_dens, h->d_dep, h->d_maps, h->d_mask_maps, h->d_err,
-                  h->d_sched, h->d_sums};
+    void *ps[] = {h->d_arena, h->d_tile_lat, h->d_masks, h->d_sched};
     for (void *p : ps)
         if (p) cudaFree(p);
     for (cudaGraphExec_t g : h->graph)
@@ -210,11 +228,14 @@ static bool valid_params(const lbm_params &p, std::string &why) {
 }
 
 // The address under which this device reads a caller's array, or null if
-// it cannot (pageable host memory, another device's memory): pinned or
-// registered host memory is mapped into the device's address space (its
-// device pointer), managed memory and this device's memory are used as
-// they are.
-static const void *device_view(const void *p) {
+// it cannot: pinned or registered host memory is mapped into the device's
+// address space (its device pointer), managed memory and this device's
+// memory are used as they are, and so is pageable host memory where the
+// device walks the host's page tables (pageable; it then reads such memory
+// at the link's rate, where a copy per array cost 1.6 ms for the 128 arrays
+// of 32 capillaries).  Null: another device's memory, or pageable memory on
+// a device that cannot address it.
+static const void *device_view(const void *p, bool pageable) {
     if (!p) return nullptr;
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -231,8 +252,19 @@ static const void *device_view(const void *p) {
     case cudaMemoryTypeManaged:
         return a.devicePointer ? a.devicePointer : p;
     default:
-        return nullptr;
+        return pageable ? p : nullptr;
     }
+}
+// Whether this device addresses pageable host memory as the host does.
+static bool reads_pageable() {
+    int dev = 0, on = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&on, cudaDevAttrPageableMemoryAccessUsesHostPageTables,
+                               dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return on != 0;
 }
 
 static void pick_tile(lbm_handle *h, const lbm_geometry *g) {
@@ -300,7 +332,8 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 // lattice's planes of 32-bit words including the ghost band (box = the
 // kernel's tile plus halo, all planes), and one over the lattice's own nodes
 // (box = the tile) for the output stores; coordinates beyond read as zeros.
-static bool make_maps(lbm_handle *h, std::string &why) {
+// (`up` holds what is uploaded; the caller keeps it until the stream has it.)
+static bool make_maps(lbm_handle *h, std::vector<CUtensorMap> &up, std::string &why) {
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (!enc) {
         why = "cuTensorMapEncodeTiled unavailable";
@@ -308,7 +341,8 @@ static bool make_maps(lbm_handle *h, std::string &why) {
     }
     const int count = h->count;
     const size_t esz = 4;
-    std::vector<CUtensorMap> maps(4 * count);
+    up.resize(5 * (size_t)count);
+    CUtensorMap *maps = up.data(), *mmaps = maps + 4 * (size_t)count;
     const cuuint64_t npl = h->half ? NW16 : NPOP;
     const CUtensorMapDataType pty = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     for (int b = 0; b < 2; ++b) {
@@ -347,7 +381,6 @@ static bool make_maps(lbm_handle *h, std::string &why) {
             }
         }
     }
-    std::vector<CUtensorMap> mmaps(count);
     for (int l = 0; l < count; ++l) {
         const LatDesc &d = h->desc[l];
         cuuint64_t dims[2] = {(cuuint64_t)d.pitch, (cuuint64_t)(d.ny + 2 * GHOST)};
@@ -366,15 +399,8 @@ static bool make_maps(lbm_handle *h, std::string &why) {
             return false;
         }
     }
-    if (cudaMalloc(&h->d_mask_maps, mmaps.size() * sizeof(CUtensorMap)) != cudaSuccess ||
-        cudaMemcpy(h->d_mask_maps, mmaps.data(), mmaps.size() * sizeof(CUtensorMap),
-                   cudaMemcpyHostToDevice) != cudaSuccess) {
-        why = "tensor map upload";
-        return false;
-    }
-    if (cudaMalloc(&h->d_maps, maps.size() * sizeof(CUtensorMap)) != cudaSuccess ||
-        cudaMemcpy(h->d_maps, maps.data(), maps.size() * sizeof(CUtensorMap),
-                   cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (cudaMemcpyAsync(h->d_maps, up.data(), up.size() * sizeof(CUtensorMap),
+                        cudaMemcpyHostToDevice, h->stream) != cudaSuccess) {
         why = "tensor map upload";
         return false;
     }
@@ -468,7 +494,7 @@ static size_t deal_tiles(const int32_t *nx, const int32_t *ny, int count,
     return slots;
 }
 
-static bool make_schedule(lbm_handle *h, std::string &why) {
+static bool make_schedule(lbm_handle *h, std::vector<TileRec> &sched, std::string &why) {
     int grid = 0;
     cudaError_t e = grid_step_tma(h->tx, h->ty, h->store(), &grid);
     if (e != cudaSuccess || grid <= 0) {
@@ -480,17 +506,35 @@ static bool make_schedule(lbm_handle *h, std::string &why) {
         nx[l] = h->desc[l].nx;
         ny[l] = h->desc[l].ny;
     }
-    std::vector<TileRec> sched;
     const size_t slots = deal_tiles(nx.data(), ny.data(), h->count, h->tx, h->ty, grid, sched);
     if (cudaMalloc(&h->d_sched, std::max<size_t>(sched.size(), 1) * sizeof(TileRec)) != cudaSuccess ||
-        cudaMemcpy(h->d_sched, sched.data(), sched.size() * sizeof(TileRec),
-                   cudaMemcpyHostToDevice) != cudaSuccess) {
+        cudaMemcpyAsync(h->d_sched, sched.data(), sched.size() * sizeof(TileRec),
+                        cudaMemcpyHostToDevice, h->stream) != cudaSuccess) {
         why = "schedule upload";
         return false;
     }
     h->sched_grid = grid;
     h->sched_slots = (int)slots;
     return true;
+}
+
+// The direct kernel's table of each tile's lattice, for the tile counts in
+// the descriptors.
+static cudaError_t make_tile_table(lbm_handle *h) {
+    std::vector<int32_t> tile_lat(h->ntiles);
+    for (int l = 0; l < h->count; ++l) {
+        const LatDesc &d = h->desc[l];
+        const int nt = d.tiles_x * ((d.ny + h->ty - 1) / h->ty);
+        for (int k = 0; k < nt; ++k) tile_lat[d.tile_base + k] = l;
+    }
+    if (h->d_tile_lat) cudaFree(h->d_tile_lat);
+    h->d_tile_lat = nullptr;
+    cudaError_t e = dalloc(&h->d_tile_lat, h->ntiles);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(h->d_tile_lat, tile_lat.data(), h->ntiles * sizeof(int32_t),
+                            cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    return e;
 }
 
 // Re-tiles every lattice for another step kernel or tile shape: tile
@@ -510,32 +554,22 @@ static lbm_status retile(lbm_handle *h, bool tma, int tx, int ty) {
         d.tile_base = tiles;
         tiles += d.tiles_x * ((d.ny + ty - 1) / ty);
     }
-    std::vector<int32_t> tile_lat(tiles);
-    for (int l = 0; l < h->count; ++l) {
-        const LatDesc &d = h->desc[l];
-        const int nt = d.tiles_x * ((d.ny + ty - 1) / ty);
-        for (int k = 0; k < nt; ++k) tile_lat[d.tile_base + k] = l;
-    }
     CK(h, cudaStreamSynchronize(h->stream));
-    if (h->d_tile_lat) cudaFree(h->d_tile_lat);
-    h->d_tile_lat = nullptr;
-    CK(h, dalloc(&h->d_tile_lat, tiles));
-    CK(h, cudaMemcpy(h->d_tile_lat, tile_lat.data(), tiles * sizeof(int32_t),
-                     cudaMemcpyHostToDevice));
     CK(h, cudaMemcpy(h->d_desc, h->desc.data(), h->count * sizeof(LatDesc),
                      cudaMemcpyHostToDevice));
     h->ntiles = tiles;
-    for (CUtensorMap **m : {&h->d_maps, &h->d_mask_maps}) {
-        if (*m) cudaFree(*m);
-        *m = nullptr;
-    }
     if (h->d_sched) cudaFree(h->d_sched);
     h->d_sched = nullptr;
     if (tma) {
         std::string why;
-        if (!make_maps(h, why) || !make_schedule(h, why))
+        std::vector<CUtensorMap> maps;
+        std::vector<TileRec> sched;
+        if (!make_maps(h, maps, why) || !make_schedule(h, sched, why))
             return fail(h, LBM_EINVAL, "tile shape not supported: " + why);
+        CK(h, cudaStreamSynchronize(h->stream));
+        return LBM_OK;
     }
+    CK(h, make_tile_table(h));
     return LBM_OK;
 }
 
@@ -626,43 +660,52 @@ extern "C" lbm_status lbm_create_batch(const lbm_geometry *g,
     h->ncols = cols;
     h->nsec = sec;
 
-    std::vector<int32_t> tile_lat(tiles), col_lat(cols);
+    // prefixes over the lattices (count + 1 entries each): nodes (staging
+    // offsets), rows, rows with the ghost band, section columns
+    const int C1 = count + 1;
+    std::vector<int64_t> pre_h(4 * C1, 0);
     for (int l = 0; l < count; ++l) {
-        const LatDesc &d = h->desc[l];
-        const int nt = d.tiles_x * ((d.ny + h->ty - 1) / h->ty);
-        for (int k = 0; k < nt; ++k) tile_lat[d.tile_base + k] = l;
-        for (int x = 0; x < d.nx; ++x) col_lat[h->col_base[l] + x] = l;
+        pre_h[l + 1] = h->in_off_host[l + 1];
+        pre_h[C1 + l + 1] = pre_h[C1 + l] + h->desc[l].ny;
+        pre_h[2 * C1 + l + 1] = pre_h[2 * C1 + l] + h->desc[l].ny + 2 * GHOST;
+        pre_h[3 * C1 + l] = h->desc[l].col_off;
     }
-    // mask bytes, section-column counts and initial wall thicknesses are
-    // built on the device from each lattice's solid array (k_mask_init,
-    // k_col_init) below
+    pre_h[3 * C1 + count] = h->nsec;
+    h->total_rows = pre_h[C1 + count];
 
-    // ---- device allocations ----------------------------------------------
+    // ---- device allocation ------------------------------------------------
     const size_t esz = 4;  // 32-bit words in both storages
-    cudaError_t e = cudaSuccess;
-#define AL(ptr, n)                                                      \
-    if (e == cudaSuccess) e = dalloc(&(ptr), (n));
-    AL(h->d_desc, count);
-    AL(h->d_tile_lat, tiles);
-    AL(h->d_col_lat, cols);
-    AL(h->d_col_base, count);
-    AL(h->d_in_off, 2 * (count + 1));
-    if (e == cudaSuccess) e = cudaMalloc(&h->d_pop[0], pop * esz);
-    if (e == cudaSuccess) e = cudaMalloc(&h->d_pop[1], pop * esz);
-    AL(h->d_mask, node);
-    AL(h->d_m, node);
-    AL(h->d_col_fluid, sec);
-    AL(h->d_wall0, 2 * sec);
-    AL(h->d_st, count);
-    AL(h->d_step, 2);
-    AL(h->d_cols, cols);
-    if (e == cudaSuccess) e = cudaMalloc(&h->d_obs, count * sizeof(lbm_obs));
-    AL(h->d_sums, 3 * count);
-    AL(h->d_canon, NPOP * h->max_nodes);
-    AL(h->d_dens, 3 * h->max_nodes);
-    AL(h->d_dep, h->max_nodes);
-    AL(h->d_err, 1);
-#undef AL
+    const int64_t total = h->in_off_host.back();
+    Arena ar;
+    // zeroed in one go
+    uint32_t *pop_w[2];
+    ar.add(&pop_w[0], (size_t)pop);
+    ar.add(&pop_w[1], (size_t)pop);
+    ar.add(&h->d_mask, (size_t)node);
+    ar.add(&h->d_m, (size_t)node);
+    ar.add(&h->d_step, 2);
+    ar.add(&h->d_err, 1);
+    const size_t zeroed = ar.bytes;
+    // uploaded in one go
+    int64_t *pre = nullptr;
+    const size_t tab = ar.bytes;
+    const size_t at_desc = ar.add(&h->d_desc, count) - tab;
+    const size_t at_col_lat = ar.add(&h->d_col_lat, cols) - tab;
+    const size_t at_col_base = ar.add(&h->d_col_base, count) - tab;
+    const size_t at_pre = ar.add(&pre, 4 * C1) - tab;
+    const size_t at_st = ar.add(&h->d_st, count) - tab;
+    const size_t tab_bytes = ar.bytes - tab;
+    ar.add(&h->d_maps, 5 * (size_t)count);
+    ar.add(&h->d_col_fluid, sec);
+    ar.add(&h->d_wall0, 2 * sec);
+    ar.add(&h->d_cols, cols);
+    lbm_obs *obs = nullptr;
+    ar.add(&obs, count);
+    ar.add(&h->d_sums, 3 * (size_t)count);
+    ar.add(&h->d_canon, NPOP * h->max_nodes);
+    ar.add(&h->d_dens, 3 * h->max_nodes);
+    ar.add(&h->d_dep, h->max_nodes);
+    cudaError_t e = ar.place(&h->d_arena);
     if (e != cudaSuccess) {
         std::string msg = std::string("device allocation: ") + cudaGetErrorString(e);
         free_all(h);
@@ -670,6 +713,11 @@ extern "C" lbm_status lbm_create_batch(const lbm_geometry *g,
         cudaGetLastError();
         return fail(nullptr, e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA, msg);
     }
+    h->d_pop[0] = pop_w[0];
+    h->d_pop[1] = pop_w[1];
+    h->d_obs = obs;
+    h->d_in_off = pre;
+    h->d_mask_maps = h->d_maps + 4 * (size_t)count;
     lbm_status st = LBM_OK;
     auto bad = [&](cudaError_t ce, const char *what) {
         if (ce != cudaSuccess && st == LBM_OK) {
@@ -680,49 +728,58 @@ extern "C" lbm_status lbm_create_batch(const lbm_geometry *g,
     bad(cudaStreamCreateWithFlags(&h->own, cudaStreamNonBlocking), "stream");
     h->stream = h->own;
     cudaStream_t s = h->stream;
+    // the zeroed buffers on a stream of their own, behind nothing, so that
+    // they run beside the gather
+    cudaStream_t s2 = nullptr;
+    cudaEvent_t zero_done = nullptr;
+    bad(cudaStreamCreateWithFlags(&s2, cudaStreamNonBlocking), "stream");
+    bad(cudaEventCreateWithFlags(&zero_done, cudaEventDisableTiming), "event");
+    if (st == LBM_OK) {
+        bad(cudaMemsetAsync(h->d_arena, 0, zeroed, s2), "memset");
+        bad(cudaEventRecord(zero_done, s2), "event");
+    }
+    // tables the kernels read
+    std::vector<uint8_t> tabs(tab_bytes, 0);
+    memcpy(&tabs[at_desc], h->desc.data(), count * sizeof(LatDesc));
+    int32_t *col_lat = reinterpret_cast<int32_t *>(&tabs[at_col_lat]);
+    for (int l = 0; l < count; ++l)
+        for (int x = 0; x < h->desc[l].nx; ++x) col_lat[h->col_base[l] + x] = l;
+    memcpy(&tabs[at_col_base], h->col_base.data(), count * sizeof(int64_t));
+    memcpy(&tabs[at_pre], pre_h.data(), pre_h.size() * sizeof(int64_t));
+    for (int l = 0; l < count; ++l)
+        reinterpret_cast<LatState *>(&tabs[at_st])[l].closure = ~0ull;
+    if (st == LBM_OK)
+        bad(cudaMemcpyAsync((char *)h->d_arena + tab, tabs.data(), tab_bytes,
+                            cudaMemcpyHostToDevice, s),
+            "tables");
     // Initial state of the whole batch: every lattice's inputs go into one
     // device staging area -- read in place by one gather kernel where the
-    // device can address the caller's arrays (pinned or registered host
-    // memory, device or managed memory), else copied by the host (one copy
-    // per pageable array) -- issued on the handle's stream and landing
-    // while the host builds the tensor maps and the schedule below; then
-    // one launch per set-up kernel covers all lattices.
-    const int64_t total = h->in_off_host.back();
+    // device can address the caller's arrays, else copied by the host (one
+    // copy per array) -- issued on the handle's stream and landing while the
+    // host builds the tensor maps and the schedule below; then one launch per
+    // set-up kernel covers all lattices.  (Mask bytes, section-column counts
+    // and initial wall thicknesses are built on the device from the solid
+    // arrays.)
     float *rho3 = nullptr;
     uint8_t *sol = nullptr;
-    // prefixes over the lattices (count + 1 entries each): nodes (staging
-    // offsets), rows, rows with the ghost band, section columns
-    const int C1 = count + 1;
-    int64_t *pre = nullptr;
-    if (st == LBM_OK) {
-        bad(dalloc(&rho3, 3 * (size_t)total), "alloc");
-        bad(dalloc(&sol, (size_t)total), "alloc");
-        bad(dalloc(&pre, 4 * (size_t)C1), "alloc");
-    }
-    std::vector<int64_t> pre_h(4 * C1, 0);
-    for (int l = 0; l < count; ++l) {
-        pre_h[l + 1] = h->in_off_host[l + 1];
-        pre_h[C1 + l + 1] = pre_h[C1 + l] + h->desc[l].ny;
-        pre_h[2 * C1 + l + 1] = pre_h[2 * C1 + l] + h->desc[l].ny + 2 * GHOST;
-        pre_h[3 * C1 + l] = h->desc[l].col_off;
-    }
-    pre_h[3 * C1 + count] = h->nsec;
-    h->total_rows = pre_h[C1 + count];
-    if (st == LBM_OK) {
-        bad(cudaMemcpyAsync(pre, pre_h.data(), pre_h.size() * 8, cudaMemcpyHostToDevice, s), "prefix");
-        bad(cudaMemcpyAsync(h->d_in_off, pre_h.data(), 2 * C1 * 8, cudaMemcpyHostToDevice, s), "prefix");
-    }
     InPtrs *d_ptrs = nullptr;
+    void *staging = nullptr;
+    Arena sg;
+    sg.add(&rho3, 3 * (size_t)total);
+    sg.add(&sol, (size_t)total);
+    sg.add(&d_ptrs, (size_t)count);
+    if (st == LBM_OK) bad(sg.place(&staging), "alloc");
+    std::vector<InPtrs> ptrs(count);
+    const bool pageable = reads_pageable();
     if (st == LBM_OK) {
-        std::vector<InPtrs> ptrs(count);
         bool any = false;
         for (int l = 0; l < count && st == LBM_OK; ++l) {
             const int64_t N = (int64_t)h->desc[l].nx * h->desc[l].ny, o = h->in_off_host[l];
             InPtrs &q = ptrs[l];
-            q.rho_a = static_cast<const float *>(device_view(g[l].rho_a));
-            q.rho_b = static_cast<const float *>(device_view(g[l].rho_b));
-            q.conc = static_cast<const float *>(device_view(g[l].conc));
-            q.solid = static_cast<const uint8_t *>(device_view(g[l].solid));
+            q.rho_a = static_cast<const float *>(device_view(g[l].rho_a, pageable));
+            q.rho_b = static_cast<const float *>(device_view(g[l].rho_b, pageable));
+            q.conc = static_cast<const float *>(device_view(g[l].conc, pageable));
+            q.solid = static_cast<const uint8_t *>(device_view(g[l].solid, pageable));
             any = any || q.rho_a || q.rho_b || q.conc || q.solid;
             // (the copy direction is inferred: pageable host memory, or
             // another device's memory)
@@ -736,10 +793,8 @@ extern "C" lbm_status lbm_create_batch(const lbm_geometry *g,
                 bad(cudaMemcpyAsync(sol + o, g[l].solid, N, cudaMemcpyDefault, s), "solid");
         }
         if (any && st == LBM_OK) {
-            bad(dalloc(&d_ptrs, (size_t)count), "alloc");
-            if (st == LBM_OK)
-                bad(cudaMemcpyAsync(d_ptrs, ptrs.data(), count * sizeof(InPtrs),
-                                    cudaMemcpyHostToDevice, s), "pointers");
+            bad(cudaMemcpyAsync(d_ptrs, ptrs.data(), count * sizeof(InPtrs),
+                                cudaMemcpyHostToDevice, s), "pointers");
             // at most 65535 lattices per launch (grid y)
             for (int l0 = 0; l0 < count && st == LBM_OK; l0 += 65535) {
                 const unsigned ny_ = (unsigned)std::min(count - l0, 65535);
@@ -749,42 +804,19 @@ extern "C" lbm_status lbm_create_batch(const lbm_geometry *g,
             }
         }
     }
-    // tables the kernels read (small synchronous copies on the legacy
-    // stream, which the handle's stream does not wait for)
-    bad(cudaMemcpy(h->d_desc, h->desc.data(), count * sizeof(LatDesc), cudaMemcpyHostToDevice), "desc");
-    bad(cudaMemcpy(h->d_tile_lat, tile_lat.data(), tiles * sizeof(int32_t), cudaMemcpyHostToDevice), "tiles");
-    bad(cudaMemcpy(h->d_col_lat, col_lat.data(), cols * sizeof(int32_t), cudaMemcpyHostToDevice), "cols");
-    bad(cudaMemcpy(h->d_col_base, h->col_base.data(), count * sizeof(int64_t), cudaMemcpyHostToDevice), "colbase");
-    std::vector<LatState> st0(count);
-    for (auto &x : st0) {
-        memset(&x, 0, sizeof(x));
-        x.closure = ~0ull;
-    }
-    bad(cudaMemcpy(h->d_st, st0.data(), count * sizeof(LatState), cudaMemcpyHostToDevice), "state");
-    // the zeroed buffers on a stream of their own, behind nothing, so that
-    // they run beside the gather; the host meanwhile builds the tensor maps
-    // and the block schedule
-    cudaStream_t s2 = nullptr;
-    bad(cudaStreamCreateWithFlags(&s2, cudaStreamNonBlocking), "stream");
-    if (st == LBM_OK) {
-        bad(cudaMemsetAsync(h->d_mask, 0, node, s2), "memset");
-        bad(cudaMemsetAsync(h->d_pop[0], 0, pop * esz, s2), "memset");
-        bad(cudaMemsetAsync(h->d_pop[1], 0, pop * esz, s2), "memset");
-        bad(cudaMemsetAsync(h->d_m, 0, node * sizeof(double), s2), "memset");
-        bad(cudaMemsetAsync(h->d_step, 0, 2 * sizeof(int64_t), s2), "memset");
-        bad(cudaMemsetAsync(h->d_err, 0, sizeof(int), s2), "memset");
-    }
+    std::vector<CUtensorMap> maps;
+    std::vector<TileRec> sched;
     if (st == LBM_OK && h->use_tma) {
         std::string why;
-        if (!make_maps(h, why) || !make_schedule(h, why)) {
+        if (!make_maps(h, maps, why) || !make_schedule(h, sched, why)) {
             g_create_err = why;
             st = LBM_ECUDA;
         }
+    } else if (st == LBM_OK) {
+        bad(make_tile_table(h), "tiles");
     }
-    // the gather (handle's stream), the zeroing (s2) and the legacy-stream
-    // copies all land before the set-up kernels
-    if (st == LBM_OK) bad(cudaDeviceSynchronize(), "sync");
-    if (s2) cudaStreamDestroy(s2);
+    // the zeroing lands before the set-up kernels
+    if (st == LBM_OK) bad(cudaStreamWaitEvent(s, zero_done, 0), "sync");
     if (st == LBM_OK) {
         k_mask_init_all<<<(unsigned)pre_h[2 * C1 + count], 128, 0, s>>>(
             h->d_desc, count, pre + 2 * C1, pre, sol, h->d_mask);
@@ -796,11 +828,12 @@ extern "C" lbm_status lbm_create_batch(const lbm_geometry *g,
             h->d_desc, count, pre + C1, pre, rho3, h->d_mask, h->d_pop[0], h->half);
         bad(cudaGetLastError(), "init kernels");
     }
-    bad(cudaStreamSynchronize(s), "init sync");
-    if (rho3) cudaFree(rho3);
-    if (sol) cudaFree(sol);
-    if (pre) cudaFree(pre);
-    if (d_ptrs) cudaFree(d_ptrs);
+    // (also after a failure: what was issued reads the arrays above)
+    if (s2) bad(cudaStreamSynchronize(s2), "init sync");
+    if (s) bad(cudaStreamSynchronize(s), "init sync");
+    if (zero_done) cudaEventDestroy(zero_done);
+    if (s2) cudaStreamDestroy(s2);
+    if (staging) cudaFree(staging);
     if (st != LBM_OK) {
         free_all(h);
         delete h;

@@ -152,6 +152,15 @@ def _params(p, precision: int) -> Params:
     return Params(*_param_values(p), int(precision))
 
 
+def _fresh(shape, dtype) -> np.ndarray:
+    """An array for a read-back, its pages present: the device's copy into
+    pages that the host has not touched yet faults on each of them (up to 12
+    ms for 12.6 MB instead of 0.11; touching them first 0.035)."""
+    out = np.empty(shape, dtype)
+    out.reshape(-1).view(np.uint8)[::4096] = 0
+    return out
+
+
 #: Geometry and Params as numpy records (the same bytes)
 GEOM_DTYPE = np.dtype([("nx", np.int32), ("ny", np.int32), ("solid", np.uintp),
                        ("rho_a", np.uintp), ("rho_b", np.uintp),
@@ -273,7 +282,7 @@ class Solver:
 
     def solid_mask(self, k: int = 0) -> np.ndarray:
         ny, nx = self.shapes[k]
-        out = np.zeros((ny, nx), np.uint8)
+        out = _fresh((ny, nx), np.uint8)
         self._check(self._lib.lbm_get_solid_mask(
             self._h, k, out.ctypes.data_as(C.POINTER(C.c_uint8)), out.size))
         return out
@@ -285,7 +294,7 @@ class Solver:
         runs at the link's full rate)."""
         sizes = [ny * nx for ny, nx in self.shapes]
         if out is None:
-            buf = np.empty(sum(sizes), np.uint8)
+            buf = _fresh(sum(sizes), np.uint8)
         else:
             buf = out.reshape(-1)
             if (buf.dtype != np.uint8 or buf.size != sum(sizes)
@@ -304,7 +313,7 @@ class Solver:
         """Post-streaming populations (22, ny, nx): A 0-8, B 9-17, solute
         18-21."""
         ny, nx = self.shapes[k]
-        out = np.zeros((NPOP, ny, nx), np.float32)
+        out = _fresh((NPOP, ny, nx), np.float32)
         self._check(self._lib.lbm_get_fields(self._h, k, FIELD_POPS,
                                              out.ctypes.data, out.nbytes))
         return out
@@ -312,14 +321,14 @@ class Solver:
     def densities(self, k: int = 0) -> np.ndarray:
         """(3, ny, nx): rho_A, rho_B, C of the post-streaming state."""
         ny, nx = self.shapes[k]
-        out = np.zeros((3, ny, nx), np.float32)
+        out = _fresh((3, ny, nx), np.float32)
         self._check(self._lib.lbm_get_fields(self._h, k, FIELD_DENSITY,
                                              out.ctypes.data, out.nbytes))
         return out
 
     def deposit(self, k: int = 0) -> np.ndarray:
         ny, nx = self.shapes[k]
-        out = np.zeros((ny, nx), np.float64)
+        out = _fresh((ny, nx), np.float64)
         self._check(self._lib.lbm_get_fields(self._h, k, FIELD_DEPOSIT,
                                              out.ctypes.data, out.nbytes))
         return out
