@@ -573,10 +573,15 @@ size_t net_smem(const lbm_mlp *h, int mt) {
     return (size_t)2 * 16 * mt * row_len(h) * sizeof(__nv_bfloat16);
 }
 
-// 16-row units per block.
-int pick_mt(const lbm_mlp *h, int batch) {
+// 16-row units per block.  Small blocks cut the latency of a pass, which every
+// block pays in full (one block: 10.3 us forward with 16 rows, 14.4 with 32,
+// 20.7 with 64), until the blocks no longer run at once: 16 rows while each SM
+// has one block, 32 while it has one (training) or two (inference, which fits
+// two at 128 registers: 8192 rows 19.1 us with 32, 21.5 with 64, 35.3 with
+// 16; a training step on 8192 rows 97.6 with 32, 88.6 with 64).
+int pick_mt(const lbm_mlp *h, int batch, bool train) {
     const int sms = 152;
-    int mt = batch <= 16 * sms ? 1 : batch <= 32 * sms ? 2 : 4;
+    int mt = batch <= 16 * sms ? 1 : batch <= 32 * sms * (train ? 1 : 2) ? 2 : 4;
     while (mt > 1 && net_smem(h, mt) > (size_t)kSmemMax) mt >>= 1;
     return mt;
 }
@@ -584,7 +589,7 @@ int pick_mt(const lbm_mlp *h, int batch) {
 template <bool TRAIN>
 cudaError_t launch_net(lbm_mlp *h, const float *x, const float *target, int batch,
                        float *y, float inv_count, int *blocks) {
-    const int mt = pick_mt(h, batch);
+    const int mt = pick_mt(h, batch, TRAIN);
     const int grid = std::min((batch + 16 * mt - 1) / (16 * mt), kMaxBlocks);
     const size_t sm = net_smem(h, mt);
     *blocks = grid;
