@@ -21,8 +21,9 @@
 namespace lbmmlp {
 
 constexpr int kMaxLayers = 9;      // L hidden + output
-constexpr int kNetThreads = 256;   // 8 warps side by side along the units
-constexpr int kNetWarps = kNetThreads / 32;
+// warps of a k_net block, side by side along the units: 16 for 16 rows, where
+// latency is all there is, else 8
+__host__ __device__ constexpr int net_warps(int mt) { return mt == 1 ? 16 : 8; }
 constexpr int kMaxBlocks = 608;    // most blocks of k_net (4 x 152 SMs)
 constexpr int DT = 64, DR = 64;    // k_dweight: tile side, batch rows a stage
 constexpr int DLD = DT + 8;        // padded row
@@ -97,16 +98,18 @@ __device__ __forceinline__ void st_bf2(__nv_bfloat16 *p, float a, float b) {
 // before the current one's epilogue.
 template <int MT, int PF>
 struct Product {
+    static constexpr int NW = net_warps(MT);
+    static constexpr int TW = 32 / NW;  // most tiles of a warp
     const uint4 *bp;  // this lane's words of the warp's first tile
-    int kt, cnt;      // words of 32 inputs; tiles of this warp, 0..4
+    int kt, cnt;      // words of 32 inputs; tiles of this warp, 0..TW
     int n0;           // first column of the warp
-    uint4 q[PF][4];
+    uint4 q[PF][TW];
 
     __device__ __forceinline__ void start(const __nv_bfloat16 *wp, int K, int N,
                                           int pass, int warp, int lane) {
         kt = pad32(K) >> 5;
         const int left = min(32, (pad32(N) >> 3) - 32 * pass);
-        const int ntw = (left + kNetWarps - 1) / kNetWarps;
+        const int ntw = (left + NW - 1) / NW;
         const int t0 = 32 * pass + warp * ntw;
         cnt = max(0, min(ntw, left - warp * ntw));
         n0 = 8 * t0;
@@ -117,15 +120,15 @@ struct Product {
     __device__ __forceinline__ void load(int p, int k) {
         if (k >= kt) return;
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < TW; ++j)
             if (j < cnt) q[p][j] = __ldg(bp + ((long)j * kt + k) * 32);
     }
     __device__ __forceinline__ void run(const __nv_bfloat16 *as, int ld, int lane,
-                                        float acc[MT][4][4]) {
+                                        float acc[MT][TW][4]) {
 #pragma unroll
         for (int mi = 0; mi < MT; ++mi)
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
+            for (int j = 0; j < TW; ++j)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) acc[mi][j][e] = 0.f;
         if (cnt == 0) return;
@@ -141,7 +144,7 @@ struct Product {
                     for (int mi = 0; mi < MT; ++mi)
                         ldsm4(af[mi], ap + mi * 16 * ld + (k0 + p) * 32 + s * 16);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
+                    for (int j = 0; j < TW; ++j)
                         if (j < cnt) {
                             const unsigned b0 = s ? q[p][j].z : q[p][j].x;
                             const unsigned b1 = s ? q[p][j].w : q[p][j].y;
@@ -160,12 +163,13 @@ struct Product {
 // every pre-activation (in BF16 for k_dweight) and the block's share of the
 // bias gradients and of the loss; without it y receives the output.
 template <int MT, bool TRAIN>
-__global__ void __launch_bounds__(kNetThreads)
+__global__ void __launch_bounds__(32 * net_warps(MT))
     k_net(const __grid_constant__ Net net, const float *__restrict__ x,
           const float *__restrict__ target, int batch, float *__restrict__ y,
           int ld, float inv_count) {
     constexpr int BM = 16 * MT;
-    constexpr int PF = MT == 1 ? 6 : MT == 2 ? 4 : 3;
+    constexpr int PF = MT == 1 ? 8 : MT == 2 ? 4 : 3;
+    constexpr int NT = 32 * net_warps(MT), TW = 32 / net_warps(MT);
     extern __shared__ __align__(16) __nv_bfloat16 sm[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = lane >> 2, t4 = lane & 3;
@@ -173,7 +177,7 @@ __global__ void __launch_bounds__(kNetThreads)
     __nv_bfloat16 *cur = sm, *nxt = sm + BM * ld;
     double lsum = 0.0;
     Product<MT, PF> pr;
-    float acc[MT][4][4];
+    float acc[MT][TW][4];
 
     for (int tile = blockIdx.x; tile * BM < batch; tile += gridDim.x) {
         const int m0 = tile * BM;
@@ -181,7 +185,7 @@ __global__ void __launch_bounds__(kNetThreads)
         pr.start(net.wf + net.off_f[0], net.dim[0], net.dim[1], 0, warp, lane);
         {  // the inputs, rounded to BF16, zero beyond the batch and n_in
             const int n_in = net.dim[0], kp = pad32(n_in);
-            for (int e = tid; e < BM * kp; e += kNetThreads) {
+            for (int e = tid; e < BM * kp; e += NT) {
                 const int r = e / kp, c = e - r * kp;
                 const bool in = c < n_in && m0 + r < batch;
                 const __nv_bfloat16 v =
@@ -206,7 +210,7 @@ __global__ void __launch_bounds__(kNetThreads)
                 else if (TRAIN && L > 0)
                     pr.start(net.wt + net.off_t[L], N, net.dim[L], 0, warp, lane);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < TW; ++j) {
                     if (j >= cnt) break;
                     const int n = n0 + 8 * j + 2 * t4;
                     const float b0 = n < N ? bias[n] : 0.f;
@@ -287,7 +291,7 @@ __global__ void __launch_bounds__(kNetThreads)
                     else if (l > 1)
                         pr.start(net.wt + net.off_t[l - 1], N, net.dim[l - 1], 0, warp, lane);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
+                    for (int j = 0; j < TW; ++j) {
                         if (j >= cnt) break;
                         const int n = n0 + 8 * j + 2 * t4;
                         float d0 = 0.f, d1 = 0.f;
@@ -329,14 +333,14 @@ __global__ void __launch_bounds__(kNetThreads)
         }
     }
     if constexpr (TRAIN) {
-        __shared__ double sl[kNetWarps];
+        __shared__ double sl[net_warps(MT)];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
         if (lane == 0) sl[warp] = lsum;
         __syncthreads();
         if (tid == 0) {
             double s = 0.0;
-            for (int v = 0; v < kNetWarps; ++v) s += sl[v];
+            for (int v = 0; v < net_warps(MT); ++v) s += sl[v];
             net.loss[blockIdx.x] = s;
         }
     }
@@ -595,11 +599,11 @@ cudaError_t launch_net(lbm_mlp *h, const float *x, const float *target, int batc
     *blocks = grid;
     const int ld = row_len(h);
     if (mt == 1)
-        k_net<1, TRAIN><<<grid, kNetThreads, sm, h->stream>>>(h->net, x, target, batch, y, ld, inv_count);
+        k_net<1, TRAIN><<<grid, 32 * net_warps(1), sm, h->stream>>>(h->net, x, target, batch, y, ld, inv_count);
     else if (mt == 2)
-        k_net<2, TRAIN><<<grid, kNetThreads, sm, h->stream>>>(h->net, x, target, batch, y, ld, inv_count);
+        k_net<2, TRAIN><<<grid, 32 * net_warps(2), sm, h->stream>>>(h->net, x, target, batch, y, ld, inv_count);
     else
-        k_net<4, TRAIN><<<grid, kNetThreads, sm, h->stream>>>(h->net, x, target, batch, y, ld, inv_count);
+        k_net<4, TRAIN><<<grid, 32 * net_warps(4), sm, h->stream>>>(h->net, x, target, batch, y, ld, inv_count);
     return cudaGetLastError();
 }
 
