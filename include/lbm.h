@@ -180,8 +180,10 @@ lbm_status lbm_set_stream(lbm_handle *h, void *cuda_stream);
 /* Advances every lattice by n >= 0 time steps of the paper's Sec. II
  * update (collision with the Martys-Chen forces, streaming with half-way
  * bounce-back, solute advection-diffusion, surface reaction, deposit and
- * growth; readings c1-c12).  Asynchronous on the bound stream.  The last
- * step of a call (n > 0) also adds up each lattice's fluid content (rho_A,
+ * growth; readings c1-c12).  Asynchronous on the bound stream.  Calls of
+ * 24 or more steps on lattices of at most 16 tiles keep the state on chip
+ * between steps, with the same results bit for bit.  The last step of a call
+ * (n > 0) also adds up each lattice's fluid content (rho_A,
  * rho_B and C over the nodes it updates), which the next lbm_observables
  * then reads instead of every node's populations. */
 lbm_status lbm_step(lbm_handle *h, int64_t n);
@@ -247,7 +249,8 @@ typedef struct lbm_tuning {
  * implementation).  Times every supported variant (direct or TMA-staged,
  * tile shapes 32x4, 32x8, 32x16, 64x4, 64x8, 128x4) for `steps` steps on this
  * handle's own state, restores the state after each trial, and keeps the
- * fastest; every variant computes bit-identical results, so only speed
+ * fastest for the steps it launches one by one (steps on chip, see lbm_step,
+ * stay as they are); every variant computes bit-identical results, so only speed
  * differs.  Synchronizes; allocates a temporary copy of the state for the
  * trials.  out (may be NULL) receives the choice.  steps >= 1. */
 lbm_status lbm_autotune(lbm_handle *h, int32_t steps, lbm_tuning *out);

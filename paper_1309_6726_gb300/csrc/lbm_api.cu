@@ -283,28 +283,38 @@ static double solid_share(const lbm_geometry &g) {
 }
 
 static void pick_tile(lbm_handle *h, const lbm_geometry *g) {
-    // 64 x 4, two 256-thread blocks per SM: measured fastest on the batched
-    // sweep and the single capillary in both storages (us per step, 64 x 8 /
-    // 64 x 4: sweep of 40 lattices FP32 267 / 252, FP16 248 / 241; 4096 x 128
-    // FP32 22.4 / 19.8, FP16 21.6 / 19.4).  Where 32 x 4 tiles leave no SM
-    // more than one tile, a step is one tile's latency, which the smaller
-    // block shortens: 256 x 32 (64 tiles) 64 x 4 / 32 x 4: FP32 5.5 / 4.3,
-    // FP16 5.3 / 4.5; beyond (1000 x 60, 480 tiles) 5.6 / 6.6.
+    // Measured, us per step.  FP16: 64 x 4, two 256-thread blocks per SM, on
+    // every workload (sweep of 40 lattices 248 at 64 x 8, 241 at 64 x 4).
+    // FP32: the same where it wins, in lattices up to 640k nodes of batches up
+    // to 24M (64 x 8 / 64 x 4: 4096 x 128 22.4 / 19.8, sweep of 40 lattices
+    // 254 / 247, of 96 627 / 620); its stores go to 22 planes at once, and in
+    // larger planes or batches one 512-thread block of 64 x 8 with an output
+    // tile is ahead (sweep of 192 lattices 1175 / 1270, of 512 3118 / 3521;
+    // 2048 x 2048 box 137 / 154, preform 142 / 242).
     constexpr int kSms = 152;
-    h->ty = 4;
-    long long small = 0;
-    for (int l = 0; l < h->count; ++l)
-        small += (long long)((g[l].nx + 31) / 32) * ((g[l].ny + 3) / 4);
-    h->tx = small <= kSms ? 32 : 64;
-    // FP32, one lattice whose two buffers exceed L2 (129 MB) and of which a
-    // quarter or more is solid: 32 x 8, whose output tile leaves the block as
-    // whole rows, against 64 x 4's stores of the fluid nodes alone. 1024 x
-    // 1024 preform 50.6 -> 41.5 us per step; a preform that fits L2 (700 x
-    // 700) 20.8 -> 22.2, the same box without solids 40.1 -> 42.2.
-    const int64_t nodes = (int64_t)g[0].nx * g[0].ny;
-    if (h->count == 1 && !h->half && 2 * NPOP * 4 * nodes > (int64_t)129 << 20 &&
-        solid_share(g[0]) >= 0.25)
-        h->tx = 32, h->ty = 8;
+    constexpr int64_t kLargeLattice = 640000, kLargeBatch = 24000000;
+    int64_t small = 0, nodes = 0, most = 0;
+    for (int l = 0; l < h->count; ++l) {
+        const int64_t n = (int64_t)g[l].nx * g[l].ny;
+        small += (int64_t)((g[l].nx + 31) / 32) * ((g[l].ny + 3) / 4);
+        nodes += n;
+        most = std::max(most, n);
+    }
+    h->tx = 64;
+    h->ty = !h->half && (most > kLargeLattice || nodes > kLargeBatch) ? 8 : 4;
+    // Where 32 x 4 tiles leave no SM more than one tile, a step is one tile's
+    // latency, which the smaller block shortens: 256 x 32 (64 tiles) 64 x 4 /
+    // 32 x 4: FP32 5.5 / 4.3, FP16 5.3 / 4.5; beyond (1000 x 60, 480 tiles)
+    // 5.6 / 6.6.
+    if (small <= kSms) {
+        h->tx = 32;
+        h->ty = 4;
+    }
+    // One FP32 lattice of that size up to 1.5M nodes, a quarter or more of it
+    // solid: 32 x 8 (preform, 64 x 8 / 32 x 8: 1024 x 1024 44.8 / 40.6, 1448 x
+    // 1448 75.4 / 80.5, 2048 x 2048 142 / 170).
+    if (h->ty == 8 && h->count == 1 && nodes <= 1500000 && solid_share(g[0]) >= 0.25)
+        h->tx = 32;
     const char *e = getenv("LBM_TILE");
     if (e) {
         int a = 0, b = 0;
@@ -936,8 +946,10 @@ static cudaError_t launch_one(lbm_handle *h, bool sum) {
 // same population buffer as input.
 static const int kGraphSteps = 16;
 // Steps per cluster launch at most (a launch stays around a millisecond), and
-// the shortest call that uses them: a launch also loads and stores the state.
-static const int kClusterSteps = 512, kClusterMin = 4;
+// the shortest call that uses them: a launch also loads and stores the state,
+// about 17 us (a call of 16 steps of 256 x 32 FP32 69 us with it and 66
+// without, of 24 steps 90 and 100, of 64 steps 204 and 245).
+static const int kClusterSteps = 512, kClusterMin = 24;
 
 // Captures kGraphSteps launches starting from buffer 0 into h->graph[sum];
 // sum: the last one adds up the lattice totals.

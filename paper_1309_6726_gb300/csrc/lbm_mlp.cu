@@ -90,6 +90,17 @@ __device__ __forceinline__ void st_bf2(__nv_bfloat16 *p, float a, float b) {
     *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(a, b);
 }
 
+// Programmatic dependent launch of the inference pass: its blocks start under
+// the tail of the launch before it in the stream, let the next one start at
+// once and wait here for the previous launch to end before they touch memory
+// (256 rows forward, back to back 10.5 -> 9.0 us, 8192 rows 20.6 -> 19.0).
+// Training's three launches are plain: with the weight gradients' blocks
+// waiting on the SMs a step on 8192 rows took 102 us instead of 89.
+__device__ __forceinline__ void start_after_previous() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // One product of a block: its rows (in shared memory, K columns) times a
 // fragment-ordered matrix of N columns, in passes of up to 256 columns; warp
 // v takes `ntw` neighbouring 8-column tiles of a pass.  Every weight is read
@@ -175,6 +186,7 @@ __global__ void __launch_bounds__(32 * net_warps(MT))
     const int g = lane >> 2, t4 = lane & 3;
     const int L = net.L;
     __nv_bfloat16 *cur = sm, *nxt = sm + BM * ld;
+    if constexpr (!TRAIN) start_after_previous();
     double lsum = 0.0;
     Product<MT, PF> pr;
     float acc[MT][TW][4];
@@ -533,6 +545,7 @@ using namespace lbmmlp;
 struct lbm_mlp {
     lbm_mlp_shape sh{};
     Net net{};
+    void *arena = nullptr;  // every device buffer
     float *m1 = nullptr, *m2 = nullptr;
     double *d_loss = nullptr;
     int tiles = 0;       // k_dweight tiles of all layers
@@ -598,13 +611,22 @@ cudaError_t launch_net(lbm_mlp *h, const float *x, const float *target, int batc
     const size_t sm = net_smem(h, mt);
     *blocks = grid;
     const int ld = row_len(h);
-    if (mt == 1)
-        k_net<1, TRAIN><<<grid, 32 * net_warps(1), sm, h->stream>>>(h->net, x, target, batch, y, ld, inv_count);
-    else if (mt == 2)
-        k_net<2, TRAIN><<<grid, 32 * net_warps(2), sm, h->stream>>>(h->net, x, target, batch, y, ld, inv_count);
-    else
-        k_net<4, TRAIN><<<grid, 32 * net_warps(4), sm, h->stream>>>(h->net, x, target, batch, y, ld, inv_count);
-    return cudaGetLastError();
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.dynamicSmemBytes = sm;
+    c.stream = h->stream;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = TRAIN ? 0 : 1;  // start_after_previous
+    auto go = [&](auto *k, int warps) {
+        c.blockDim = dim3(32 * warps);
+        return cudaLaunchKernelEx(&c, k, h->net, x, target, batch, y, ld, inv_count);
+    };
+    return mt == 1   ? go(k_net<1, TRAIN>, net_warps(1))
+           : mt == 2 ? go(k_net<2, TRAIN>, net_warps(2))
+                     : go(k_net<4, TRAIN>, net_warps(4));
 }
 
 // Gradient of the loss into grad (when not null); adam: also the update.
@@ -685,15 +707,20 @@ lbm_status lbm_mlp_create(const lbm_mlp_shape *shape, lbm_mlp **out) {
     net.np = np;
     // parts of a weight gradient: about three blocks per SM
     h->max_split = std::min(std::max(456 / h->tiles, 1), 16);
-    bool ok = true;
+    // one allocation: each buffer's place in it, then the buffers
+    struct Item { void **p; size_t at; };
+    std::vector<Item> items;
+    size_t bytes = 0;
     auto al = [&](auto **p, size_t n) {
-        if (ok && cudaMalloc(p, std::max<size_t>(n, 1) * sizeof(**p)) != cudaSuccess) ok = false;
+        items.push_back({(void **)p, bytes});
+        bytes += (std::max<size_t>(n, 1) * sizeof(**p) + 255) / 256 * 256;
     };
     al(&net.w, np);
     al(&h->m1, np);
     al(&h->m2, np);
     al(&net.wf, nf);
     al(&net.wt, nt);
+    const size_t zeroed = bytes;
     for (int l = 0; l <= s.n_layers; ++l) {
         if (l < s.n_layers) al(&net.hs[l], (size_t)s.max_batch * s.n_hidden);
         al(&net.act[l], (size_t)s.max_batch * pad32(net.dim[l]));
@@ -704,14 +731,14 @@ lbm_status lbm_mlp_create(const lbm_mlp_shape *shape, lbm_mlp **out) {
     al(&net.loss, blocks);
     al(&net.parts, (size_t)h->max_split * np);
     al(&h->d_loss, 1);
+    bool ok = cudaMalloc(&h->arena, bytes) == cudaSuccess;
+    if (ok)
+        for (const Item &i : items) *i.p = (char *)h->arena + i.at;
     if (ok && cudaStreamCreateWithFlags(&h->own, cudaStreamNonBlocking) != cudaSuccess)
         ok = false;
     h->stream = h->own;
     if (ok) {
-        for (void *p : {(void *)net.w, (void *)h->m1, (void *)h->m2})
-            ok = ok && cudaMemset(p, 0, np * sizeof(float)) == cudaSuccess;
-        ok = ok && cudaMemset(net.wf, 0, nf * sizeof(__nv_bfloat16)) == cudaSuccess;
-        ok = ok && cudaMemset(net.wt, 0, nt * sizeof(__nv_bfloat16)) == cudaSuccess;
+        ok = cudaMemset(h->arena, 0, zeroed) == cudaSuccess;
         const int a = (int)cudaFuncAttributeMaxDynamicSharedMemorySize;
         for (const void *f : {(const void *)k_net<1, false>, (const void *)k_net<1, true>,
                               (const void *)k_net<2, false>, (const void *)k_net<2, true>,
@@ -795,14 +822,7 @@ lbm_status lbm_mlp_train_step(lbm_mlp *h, const float *x, const float *target,
 void lbm_mlp_destroy(lbm_mlp *h) {
     if (!h) return;
     if (h->stream) cudaStreamSynchronize(h->stream);
-    const Net &net = h->net;
-    for (void *p : {(void *)net.w, (void *)h->m1, (void *)h->m2, (void *)net.wf,
-                    (void *)net.wt, (void *)net.db, (void *)net.loss,
-                    (void *)net.parts, (void *)h->d_loss})
-        if (p) cudaFree(p);
-    for (int l = 0; l < kMaxLayers; ++l)
-        for (void *p : {(void *)net.hs[l], (void *)net.act[l], (void *)net.dz[l]})
-            if (p) cudaFree(p);
+    if (h->arena) cudaFree(h->arena);
     if (h->own) cudaStreamDestroy(h->own);
     delete h;
 }

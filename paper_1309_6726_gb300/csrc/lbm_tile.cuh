@@ -51,7 +51,8 @@ struct TmaTile {
     // For FP32 an output tile of 64 x 4 leaves room for one block only
     // (sweep of 40 lattices: one 512-thread block of 64 x 8 with an output
     // tile 267 us per step, two of 64 x 4 with direct stores 252; 4096 x 128:
-    // 22.4 and 19.8).  FP32 32 x 8 fits two blocks with its output tile, and
+    // 22.4 and 19.8; larger planes and batches the other way round, see
+    // pick_tile).  FP32 32 x 8 fits two blocks with its output tile, and
     // keeps it: slower on capillaries (308 us on the sweep) but the fastest
     // where solid nodes are everywhere (1024 x 1024 preform: 44.0 us against
     // 50.9 without it and 48.4 at 64 x 4).  (FP16: the budget of three
