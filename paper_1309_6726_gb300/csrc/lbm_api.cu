@@ -441,6 +441,49 @@ static bool make_maps(lbm_handle *h, std::vector<CUtensorMap> &up, std::string &
     return true;
 }
 
+struct Strip { int lat, col, row0, rows; };
+
+// Deals strips, longest first, to the block with the least work so far (ties
+// to the lower index).
+static void deal_strips(std::vector<Strip> &strips, int grid,
+                        std::vector<std::vector<int>> &lists,
+                        std::vector<long long> &load) {
+    std::stable_sort(strips.begin(), strips.end(),
+                     [](const Strip &a, const Strip &b) { return a.rows > b.rows; });
+    lists.assign(grid, {});
+    load.assign(grid, 0);
+    std::vector<int> heap(grid);
+    for (int b = 0; b < grid; ++b) heap[b] = b;
+    auto less = [&](int a, int b) { return load[a] > load[b] || (load[a] == load[b] && a > b); };
+    std::make_heap(heap.begin(), heap.end(), less);
+    for (size_t i = 0; i < strips.size(); ++i) {
+        std::pop_heap(heap.begin(), heap.end(), less);
+        const int b = heap.back();
+        lists[b].push_back((int)i);
+        load[b] += strips[i].rows;
+        std::push_heap(heap.begin(), heap.end(), less);
+    }
+}
+
+// The tiles of dealt strips as the kernel's table; returns the slots per block.
+static size_t lay_strips(const std::vector<Strip> &strips, int tx, int ty, int grid,
+                         const std::vector<std::vector<int>> &lists,
+                         const std::vector<long long> &load,
+                         std::vector<TileRec> &sched) {
+    size_t slots = 0;
+    for (long long n : load) slots = std::max(slots, (size_t)n);
+    sched.assign((size_t)grid * slots, TileRec{-1, 0, 0, 0});
+    for (int b = 0; b < grid; ++b) {
+        size_t k = 0;
+        for (int i : lists[b]) {
+            const Strip &st = strips[i];
+            for (int r = st.row0; r < st.row0 + st.rows; ++r)
+                sched[b + k++ * grid] = TileRec{st.lat, st.col * tx, r * ty, 0};
+        }
+    }
+    return slots;
+}
+
 // Tile schedule of the persistent TMA kernel, host arithmetic only.  A
 // strip is a run of tiles down one tile column of a lattice (the halo rows
 // each tile copies were just copied by the tile above it).  Columns taller
@@ -452,7 +495,6 @@ static bool make_maps(lbm_handle *h, std::vector<CUtensorMap> &up, std::string &
 // done).  Returns the slots per block.
 static size_t plan_tiles(const int32_t *nx, const int32_t *ny, int count,
                          int tx, int ty, int grid, std::vector<TileRec> &sched) {
-    struct Strip { int lat, col, row0, rows; };
     long long total = 0;
     for (int l = 0; l < count; ++l)
         total += (long long)((nx[l] + tx - 1) / tx) * ((ny[l] + ty - 1) / ty);
@@ -465,29 +507,10 @@ static size_t plan_tiles(const int32_t *nx, const int32_t *ny, int count,
             for (int r0 = 0; r0 < rows; r0 += (int)seg)
                 strips.push_back({l, c, r0, (int)std::min<long long>(seg, rows - r0)});
     }
-    std::stable_sort(strips.begin(), strips.end(),
-                     [](const Strip &a, const Strip &b) { return a.rows > b.rows; });
-    std::vector<std::vector<TileRec>> lists(grid);
-    std::vector<long long> load(grid, 0);
-    // blocks ordered by load with a simple binary heap
-    std::vector<int> heap(grid);
-    for (int b = 0; b < grid; ++b) heap[b] = b;
-    auto less = [&](int a, int b) { return load[a] > load[b] || (load[a] == load[b] && a > b); };
-    std::make_heap(heap.begin(), heap.end(), less);
-    for (const Strip &st : strips) {
-        std::pop_heap(heap.begin(), heap.end(), less);
-        const int b = heap.back();
-        for (int r = st.row0; r < st.row0 + st.rows; ++r)
-            lists[b].push_back(TileRec{st.lat, st.col * tx, r * ty, 0});
-        load[b] += st.rows;
-        std::push_heap(heap.begin(), heap.end(), less);
-    }
-    size_t slots = 0;
-    for (auto &v : lists) slots = std::max(slots, v.size());
-    sched.assign((size_t)grid * slots, TileRec{-1, 0, 0, 0});
-    for (int b = 0; b < grid; ++b)
-        for (size_t k = 0; k < lists[b].size(); ++k) sched[b + k * grid] = lists[b][k];
-    return slots;
+    std::vector<std::vector<int>> lists;
+    std::vector<long long> load;
+    deal_strips(strips, grid, lists, load);
+    return lay_strips(strips, tx, ty, grid, lists, load, sched);
 }
 
 // The schedule of a handle.  Batches of many tiles per block are dealt in
@@ -503,13 +526,70 @@ static size_t plan_tiles(const int32_t *nx, const int32_t *ny, int count,
 // gives: a 1024 x 1024 preform (13.5 tiles) 52.1 / 57.2 us, three 4096 x 128
 // lattices FP16 (20.2 tiles) 51.8 / 53.3 us, so the line is at 8.
 constexpr int kRunTiles = 8;  // most tiles per block dealt as runs
+// From 16 to 32 tiles per block, in lattices of at most 64 tiles a column, the
+// strips are evened out (even_strips) where that takes a sixteenth off the
+// fullest block.  us per step, plan_tiles / even_strips: three 4096 x 128
+// lattices FP32 54.9 / 51.6, FP16 50.0 / 48.5, three of 4600 x 160 FP32 76.4 /
+// 70.4, FP16 72.7 / 65.9, five of the sweep FP32 52.9 / 49.9.  Where less is to
+// be had the shorter strips cost as much (four 4096 x 128 lattices, 29 tiles
+// against 28: FP32 68.7 / 70.8, FP16 65.8 / 62.8; ten of the sweep FP32 72.8 /
+// 73.7), fewer tiles per block gain nothing (three of 3001 x 97, 11.6: FP32
+// 32.9 / 33.6), and tall lattices lose more halo sharing than the balance
+// gives (1024 x 1024 preform BF16 42.5 / 44.5).
+constexpr int kEvenFrom = 16, kEvenTo = 32, kEvenRows = 64;
+
+// As plan_tiles, but each tile column is cut into equal pieces (their lengths
+// differ by one), of the length 3 to 8 that leaves the fullest block the
+// least, the longest such.
+static size_t even_strips(const int32_t *nx, const int32_t *ny, int count, int tx,
+                          int ty, int grid, std::vector<TileRec> &sched) {
+    std::vector<Strip> strips, best;
+    std::vector<std::vector<int>> lists, best_lists;
+    std::vector<long long> load, best_load;
+    long long best_max = 0;
+    for (int seg = 8; seg >= 3; --seg) {
+        strips.clear();
+        for (int l = 0; l < count; ++l) {
+            const int cols = (nx[l] + tx - 1) / tx, rows = (ny[l] + ty - 1) / ty;
+            const int n = (rows + seg - 1) / seg;
+            for (int c = 0; c < cols; ++c)
+                for (int k = 0; k < n; ++k) {
+                    const int r0 = (int)((long long)k * rows / n);
+                    strips.push_back({l, c, r0, (int)((long long)(k + 1) * rows / n) - r0});
+                }
+        }
+        deal_strips(strips, grid, lists, load);
+        const long long top = *std::max_element(load.begin(), load.end());
+        if (best.empty() || top < best_max) {
+            best_max = top;
+            best = strips;
+            best_lists = lists;
+            best_load = load;
+        }
+    }
+    return lay_strips(best, tx, ty, grid, best_lists, best_load, sched);
+}
+
 static size_t deal_tiles(const int32_t *nx, const int32_t *ny, int count,
                          int tx, int ty, int grid, std::vector<TileRec> &sched) {
     long long total = 0;
     for (int l = 0; l < count; ++l)
         total += (long long)((nx[l] + tx - 1) / tx) * ((ny[l] + ty - 1) / ty);
-    if (total > (long long)kRunTiles * grid)
-        return plan_tiles(nx, ny, count, tx, ty, grid, sched);
+    if (total > (long long)kRunTiles * grid) {
+        const size_t slots = plan_tiles(nx, ny, count, tx, ty, grid, sched);
+        int tall = 0;
+        for (int l = 0; l < count; ++l) tall = std::max(tall, (ny[l] + ty - 1) / ty);
+        if (total > (long long)kEvenFrom * grid && total <= (long long)kEvenTo * grid &&
+            tall <= kEvenRows) {
+            std::vector<TileRec> even;
+            const size_t n = even_strips(nx, ny, count, tx, ty, grid, even);
+            if (16 * n <= 15 * slots) {
+                sched.swap(even);
+                return n;
+            }
+        }
+        return slots;
+    }
     const size_t slots = (size_t)((total + grid - 1) / grid);
     sched.assign((size_t)grid * slots, TileRec{-1, 0, 0, 0});
     // block b: tiles [first, end), end = ceil((b + 1) total / grid)
