@@ -275,8 +275,9 @@ lbm_status lbm_fit_reff(const double *t, const double *z, int32_t n,
 
 /* Tile schedule of the TMA-staged step kernel (project addition; the paper
  * describes no implementation), computed on the host as lbm_create computes
- * it for handles of more than 8 tiles per block (those with fewer deal each
- * block one run of consecutive tiles): the tiles of tx by ty nodes of `count`
+ * it for most handles of more than 8 tiles per block (those with fewer deal
+ * each block one run of consecutive tiles, and short lattices with 16 to 32
+ * may have their strips evened out): the tiles of tx by ty nodes of `count`
  * lattices of nx[l] by ny[l] nodes, dealt to `grid` persistent blocks.  A strip is a run of tiles down
  * one tile column of a lattice; columns longer than
  * max(4, ceil(tiles / (4 grid))) tiles are cut into strips of that length,
