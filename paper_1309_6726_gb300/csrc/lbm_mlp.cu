@@ -22,7 +22,8 @@ namespace lbmmlp {
 
 constexpr int kMaxLayers = 9;      // L hidden + output
 // warps of a k_net block, side by side along the units: 16 for 16 rows, where
-// latency is all there is, else 8
+// latency is all there is (8 -> 16: 256 rows forward 10.5 -> 9.1 us, a
+// training step on 1024 rows 38.3 -> 32.6), else 8
 __host__ __device__ constexpr int net_warps(int mt) { return mt == 1 ? 16 : 8; }
 constexpr int kMaxBlocks = 608;    // most blocks of k_net (4 x 152 SMs)
 constexpr int DT = 64, DR = 64;    // k_dweight: tile side, batch rows a stage
@@ -173,6 +174,11 @@ struct Product {
 // gridDim.x-th such tile after it.  TRAIN: also the loss, the gradients at
 // every pre-activation (in BF16 for k_dweight) and the block's share of the
 // bias gradients and of the loss; without it y receives the output.
+//
+// Bound by latency: the chain of products, each with 128 KB of weights from L2
+// per block, and the epilogues' tanh (tensor pipe 4 % busy in training on 1024
+// rows, 23 % forward on 8192).  One launch per product took 133 us forward on
+// 256 rows and 158 on 8192; this 9.1 and 19.0.
 template <int MT, bool TRAIN>
 __global__ void __launch_bounds__(32 * net_warps(MT))
     k_net(const __grid_constant__ Net net, const float *__restrict__ x,
@@ -368,7 +374,10 @@ __device__ __forceinline__ void cp16(void *dst, const void *src, bool in) {
 // Weight gradients of every layer, dW_l[n][k] = sum over the batch of
 // dz_l[b][n] act_l[b][k]: block x takes a DT x DT tile of one layer, block y
 // `rows` rows of the batch (a multiple of DR), and writes its part to
-// parts[y].  Both operands lie batch-major; ldmatrix transposes them.
+// parts[y].  Both operands lie batch-major; ldmatrix transposes them.  About
+// 450 blocks, each waiting for its operands from L2: 8.7 us for 1024 rows of
+// the 5-256-256-256-65 network, where the layers' products and column sums
+// took 36 and 59 us each.
 __global__ void __launch_bounds__(kDwThreads)
     k_dweight(const __grid_constant__ Net net, int batch, int rows) {
     __shared__ __align__(16) __nv_bfloat16 sa[2][DR][DLD], sb[2][DR][DLD];
@@ -475,7 +484,8 @@ __device__ __forceinline__ float adam(const Net &net, const AdamArgs &o, long i,
 // null) and, with ADAM, updates the parameters.  Blocks x < nwb take 256
 // parameters each and do the weights among them; the others take 32 bias
 // entries each, 8 threads sharing the k_net blocks' shares of an entry; the
-// last of them also adds up the loss.
+// last of them also adds up the loss.  Latency of the parts' loads: 7.8 us
+// for 149,000 parameters in 8 parts.
 template <bool ADAM>
 __global__ void __launch_bounds__(256)
     k_finish(const __grid_constant__ Net net, int split, int nblk, int nwb,
@@ -591,7 +601,7 @@ size_t net_smem(const lbm_mlp *h, int mt) {
 }
 
 // 16-row units per block.  Small blocks cut the latency of a pass, which every
-// block pays in full (one block: 10.3 us forward with 16 rows, 14.4 with 32,
+// block pays in full (one block: 8.8 us forward with 16 rows, 14.4 with 32,
 // 20.7 with 64), until the blocks no longer run at once: 16 rows while each SM
 // has one block, 32 while it has one (training) or two (inference, which fits
 // two at 128 registers: 8192 rows 19.1 us with 32, 21.5 with 64, 35.3 with
