@@ -233,10 +233,13 @@ static bool valid_params(const lbm_params &p, std::string &why) {
 // memory are used as they are, and so is pageable host memory where the
 // device walks the host's page tables (pageable; it then reads such memory
 // at the link's rate, where a copy per array cost 1.6 ms for the 128 arrays
-// of 32 capillaries).  Null: another device's memory, or pageable memory on
-// a device that cannot address it.
-static const void *device_view(const void *p, bool pageable) {
-    if (!p) return nullptr;
+// of 32 capillaries).  Null: another device's memory, pageable memory on a
+// device that cannot address it, or an address that is no multiple of the
+// element's size (a view into a byte buffer, a file mapped behind an odd
+// header): the host may read and copy such an array, a device load faults.
+template <class T>
+static const T *device_view(const T *p, bool pageable) {
+    if (!p || reinterpret_cast<uintptr_t>(p) % sizeof(T) != 0) return nullptr;
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
@@ -244,13 +247,14 @@ static const void *device_view(const void *p, bool pageable) {
     }
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    const T *mapped = static_cast<const T *>(a.devicePointer);
     switch (a.type) {
     case cudaMemoryTypeHost:
-        return a.devicePointer;
+        return mapped;
     case cudaMemoryTypeDevice:
-        return a.device == dev ? a.devicePointer : nullptr;
+        return a.device == dev ? mapped : nullptr;
     case cudaMemoryTypeManaged:
-        return a.devicePointer ? a.devicePointer : p;
+        return mapped ? mapped : p;
     default:
         return pageable ? p : nullptr;
     }
@@ -890,13 +894,13 @@ extern "C" lbm_status lbm_create_batch(const lbm_geometry *g,
         for (int l = 0; l < count && st == LBM_OK; ++l) {
             const int64_t N = (int64_t)h->desc[l].nx * h->desc[l].ny, o = h->in_off_host[l];
             InPtrs &q = ptrs[l];
-            q.rho_a = static_cast<const float *>(device_view(g[l].rho_a, pageable));
-            q.rho_b = static_cast<const float *>(device_view(g[l].rho_b, pageable));
-            q.conc = static_cast<const float *>(device_view(g[l].conc, pageable));
-            q.solid = static_cast<const uint8_t *>(device_view(g[l].solid, pageable));
+            q.rho_a = device_view(g[l].rho_a, pageable);
+            q.rho_b = device_view(g[l].rho_b, pageable);
+            q.conc = device_view(g[l].conc, pageable);
+            q.solid = device_view(g[l].solid, pageable);
             any = any || q.rho_a || q.rho_b || q.conc || q.solid;
-            // (the copy direction is inferred: pageable host memory, or
-            // another device's memory)
+            // (the copy direction is inferred: host memory, or another
+            // device's)
             if (!q.rho_a)
                 bad(cudaMemcpyAsync(rho3 + 3 * o, g[l].rho_a, N * 4, cudaMemcpyDefault, s), "rho_a");
             if (!q.rho_b)

@@ -153,8 +153,9 @@ struct NodeTot {
 
 // One lattice's input arrays (row-major ny * nx) as the device addresses
 // them: pinned or registered host memory (mapped into the device's address
-// space), managed or this device's memory.  A null entry: the host copied
-// that array into the staging area instead (pageable host memory).
+// space), managed or this device's memory, and pageable host memory where the
+// device walks the host's page tables; each a multiple of its element's size.
+// A null entry: the host copied that array into the staging area instead.
 struct InPtrs {
     const float *rho_a, *rho_b, *conc;
     const uint8_t *solid;
