@@ -748,7 +748,10 @@ lbm_status lbm_mlp_create(const lbm_mlp_shape *shape, lbm_mlp **out) {
         ok = false;
     h->stream = h->own;
     if (ok) {
-        ok = cudaMemset(h->arena, 0, zeroed) == cudaSuccess;
+        // (on the handle's stream, which the default stream's queue does not
+        // order, and waited for: the next call may come on any stream)
+        ok = cudaMemsetAsync(h->arena, 0, zeroed, h->own) == cudaSuccess &&
+             cudaStreamSynchronize(h->own) == cudaSuccess;
         const int a = (int)cudaFuncAttributeMaxDynamicSharedMemorySize;
         for (const void *f : {(const void *)k_net<1, false>, (const void *)k_net<1, true>,
                               (const void *)k_net<2, false>, (const void *)k_net<2, true>,
