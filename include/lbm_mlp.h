@@ -78,7 +78,9 @@ lbm_status lbm_mlp_get_params(lbm_mlp *h, float *host, int64_t n);
 /* Binds a CUDA stream (cudaStream_t) for every later call; NULL selects
  * the handle's own non-blocking stream (cudaStreamLegacy selects the
  * legacy default stream).  Callers that produce inputs or consume outputs
- * on another stream bind that stream first. */
+ * on another stream bind that stream first.  Work queued on the stream bound
+ * until then comes first: the new stream waits for it, unless one of the two
+ * is being captured; so a stream is destroyed only after another is bound. */
 lbm_status lbm_mlp_set_stream(lbm_mlp *h, void *cuda_stream);
 
 /* Inference: y = network(x) for `batch` rows (1 <= batch <= max_batch). */

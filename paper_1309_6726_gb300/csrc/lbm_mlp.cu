@@ -561,6 +561,7 @@ struct lbm_mlp {
     int tiles = 0;       // k_dweight tiles of all layers
     int max_split = 1;   // parts of the weight gradients
     cudaStream_t own = nullptr, stream = nullptr;
+    cudaEvent_t moved = nullptr;  // end of the work queued before a change of stream
     long adam_t = 0;
     std::string err;
     bool dead = false;
@@ -671,6 +672,15 @@ lbm_status check_batch(lbm_mlp *h, int batch) {
     return LBM_OK;
 }
 
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &c) != cudaSuccess) {  // (the legacy stream during a capture)
+        cudaGetLastError();
+        return true;
+    }
+    return c != cudaStreamCaptureStatusNone;
+}
+
 lbm_status read_loss(lbm_mlp *h, double *loss) {
     if (!loss) return LBM_OK;
     MCK(h, cudaMemcpyAsync(loss, h->d_loss, sizeof(double),
@@ -744,7 +754,8 @@ lbm_status lbm_mlp_create(const lbm_mlp_shape *shape, lbm_mlp **out) {
     bool ok = cudaMalloc(&h->arena, bytes) == cudaSuccess;
     if (ok)
         for (const Item &i : items) *i.p = (char *)h->arena + i.at;
-    if (ok && cudaStreamCreateWithFlags(&h->own, cudaStreamNonBlocking) != cudaSuccess)
+    if (ok && (cudaStreamCreateWithFlags(&h->own, cudaStreamNonBlocking) != cudaSuccess ||
+               cudaEventCreateWithFlags(&h->moved, cudaEventDisableTiming) != cudaSuccess))
         ok = false;
     h->stream = h->own;
     if (ok) {
@@ -796,7 +807,18 @@ lbm_status lbm_mlp_get_params(lbm_mlp *h, float *host, int64_t n) {
 
 lbm_status lbm_mlp_set_stream(lbm_mlp *h, void *cuda_stream) {
     if (!h) return LBM_EINVAL;
-    h->stream = cuda_stream ? static_cast<cudaStream_t>(cuda_stream) : h->own;
+    const cudaStream_t to = cuda_stream ? static_cast<cudaStream_t>(cuda_stream) : h->own;
+    if (to == h->stream) return LBM_OK;
+    // weights, moments and activations are shared by all calls: what the next
+    // ones queue on the new stream waits for what is queued on the old one.
+    // (A stream that is being captured can neither wait for work outside the
+    // capture nor be waited for from outside: there the caller orders the
+    // replays, as with any captured work.)
+    if (!h->dead && !capturing(h->stream) && !capturing(to)) {
+        MCK(h, cudaEventRecord(h->moved, h->stream));
+        MCK(h, cudaStreamWaitEvent(to, h->moved, 0));
+    }
+    h->stream = to;
     return LBM_OK;
 }
 
@@ -836,6 +858,7 @@ void lbm_mlp_destroy(lbm_mlp *h) {
     if (!h) return;
     if (h->stream) cudaStreamSynchronize(h->stream);
     if (h->arena) cudaFree(h->arena);
+    if (h->moved) cudaEventDestroy(h->moved);
     if (h->own) cudaStreamDestroy(h->own);
     delete h;
 }

@@ -46,3 +46,52 @@ def test_parameters_set_while_the_default_stream_is_busy():
     assert torch.equal(net.forward(x).cpu(), want)
     net.close()
     first.close()
+
+
+def test_calls_on_another_stream_follow_the_queued_ones():
+    import torch
+    from paper_1309_6726_gb300 import mlp
+    x, t = _data()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    got = []
+    for switch in (False, True):
+        net = mlp.Mlp(*SHAPE, max_batch=48)
+        net.set_params(_theta(net.param_count))
+        torch.cuda.synchronize()
+        with torch.cuda.stream(a):
+            net.forward(x)
+            torch.cuda._sleep(BUSY if switch else 1)
+            for _ in range(3):
+                net.train_step(x, t, 1e-2)
+        with torch.cuda.stream(b if switch else a):
+            y = net.forward(x)
+            g, loss = net.grad(x, t)
+            y, g = y.cpu(), g.cpu()
+        torch.cuda.synchronize()
+        got.append((y, g, loss, net.params()))
+        net.close()
+    assert torch.equal(got[0][0], got[1][0])
+    assert torch.equal(got[0][1], got[1][1])
+    assert got[0][2] == got[1][2]
+    np.testing.assert_array_equal(got[0][3], got[1][3])
+
+
+def test_a_captured_pass_follows_passes_on_other_streams():
+    # the capturing stream cannot wait for work outside the capture; the
+    # caller orders the replay, as with any captured work
+    import torch
+    from paper_1309_6726_gb300 import mlp
+    x, t = _data()
+    net = mlp.Mlp(*SHAPE, max_batch=48)
+    net.set_params(_theta(net.param_count))
+    want = net.forward(x)
+    out = torch.empty_like(want)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        net.forward(x, out)
+    out.zero_()
+    graph.replay()
+    assert torch.equal(out, want)
+    assert torch.equal(net.forward(x), want)
+    net.close()
