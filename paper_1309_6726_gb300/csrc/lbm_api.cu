@@ -143,6 +143,9 @@ struct lbm_handle {
 static thread_local std::string g_create_err;
 
 static lbm_status fail(lbm_handle *h, lbm_status st, const std::string &msg) {
+    // the message below reports the error: left pending it would be taken for
+    // one of the next launch, of this or of another handle
+    if (st == LBM_ECUDA || st == LBM_ENOMEM) cudaGetLastError();
     if (h) {
         h->err = msg;
         if (st == LBM_ECUDA) h->dead = true;
@@ -682,8 +685,10 @@ static lbm_status retile(lbm_handle *h, bool tma, int tx, int ty) {
         std::string why;
         std::vector<CUtensorMap> maps;
         std::vector<TileRec> sched;
-        if (!make_maps(h, maps, why) || !make_schedule(h, sched, why))
+        if (!make_maps(h, maps, why) || !make_schedule(h, sched, why)) {
+            cudaGetLastError();
             return fail(h, LBM_EINVAL, "tile shape not supported: " + why);
+        }
         CK(h, cudaStreamSynchronize(h->stream));
         return LBM_OK;
     }
@@ -828,7 +833,6 @@ extern "C" lbm_status lbm_create_batch(const lbm_geometry *g,
         std::string msg = std::string("device allocation: ") + cudaGetErrorString(e);
         free_all(h);
         delete h;
-        cudaGetLastError();
         return fail(nullptr, e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA, msg);
     }
     h->d_pop[0] = pop_w[0];
@@ -955,6 +959,7 @@ extern "C" lbm_status lbm_create_batch(const lbm_geometry *g,
     if (st != LBM_OK) {
         free_all(h);
         delete h;
+        cudaGetLastError();  // (as fail does)
         return st;
     }
     *out = h;
@@ -1450,7 +1455,6 @@ extern "C" lbm_status lbm_autotune(lbm_handle *h, int32_t steps,
     for (auto &p : parts) total += (p.bytes + 255) / 256 * 256;
     char *snap = nullptr;
     if (cudaMalloc(&snap, total) != cudaSuccess) {
-        cudaGetLastError();
         return fail(h, LBM_ENOMEM, "autotune: no room for a state copy");
     }
     auto copy_all = [&](bool save) -> cudaError_t {

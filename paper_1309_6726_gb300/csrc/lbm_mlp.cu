@@ -571,6 +571,9 @@ namespace {
 std::string g_create_err;
 
 lbm_status fail(lbm_mlp *h, lbm_status st, const std::string &msg) {
+    // the message below reports the error: left pending it would be taken for
+    // one of the next launch, of this or of another handle
+    if (st == LBM_ECUDA || st == LBM_ENOMEM) cudaGetLastError();
     if (h) {
         h->err = msg;
         if (st == LBM_ECUDA) h->dead = true;
