@@ -1345,9 +1345,13 @@ extern "C" lbm_status lbm_load(lbm_handle *h, const char *path) {
          hd.nsec == h->nsec;
     std::vector<LatDesc> dsc(h->count);
     ok = ok && fread(dsc.data(), sizeof(LatDesc), h->count, f) == (size_t)h->count;
-    if (ok) {
-        for (int l = 0; l < h->count; ++l)
-            if (memcmp(&dsc[l], &h->desc[l], sizeof(LatDesc)) != 0) ok = false;
+    // the tiles are how a handle launches, not part of the state: they depend
+    // on the storage, the sizes and the solid share at create
+    for (int l = 0; ok && l < h->count; ++l) {
+        LatDesc mine = h->desc[l];
+        mine.tiles_x = dsc[l].tiles_x;
+        mine.tile_base = dsc[l].tile_base;
+        ok = memcmp(&dsc[l], &mine, sizeof(LatDesc)) == 0;
     }
     if (!ok) {
         fclose(f);
