@@ -1068,18 +1068,24 @@ extern "C" lbm_status lbm_step(lbm_handle *h, int64_t n) {
     // The last launch of the call adds up the lattice totals of the state it
     // leaves (a replay that ends the call uses the graph whose last launch
     // sums).
-    // Lattices that fit a cluster: all but the last step on chip, up to
-    // kClusterSteps per launch.  (Not while the caller captures the stream:
-    // a launch moves the state to the other buffer whatever its step count,
-    // and a graph replayed from one buffer counts on one move per step.)
+    // Lattices that fit a cluster: all but the last steps on chip, up to
+    // kClusterSteps per launch.  A launch moves the state to the other buffer
+    // whatever its step count, and a graph that the caller captured around
+    // lbm_step reads the buffer it was captured with.  So none are captured,
+    // and a call moves the state as often as n single steps would, give or
+    // take an even number: the steps left for single launches, one to three,
+    // see to it.
     if (h->csize > 0 && h->stall_tx == 0 && n >= kClusterMin) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess) {
             cudaGetLastError();
             cap = cudaStreamCaptureStatusActive;
         }
-        while (cap == cudaStreamCaptureStatusNone && n > 1) {
-            const int m = (int)std::min<int64_t>(n - 1, kClusterSteps);
+        int64_t single = 1;
+        while (((n - single + kClusterSteps - 1) / kClusterSteps + single - n) % 2 != 0)
+            ++single;
+        while (cap == cudaStreamCaptureStatusNone && n > single) {
+            const int m = (int)std::min<int64_t>(n - single, kClusterSteps);
             CK(h, launch_step_cluster(step_args(h), h->count, m, h->ctx, h->cty,
                                       h->csize, h->store(), h->stream));
             h->cur ^= 1;
