@@ -29,6 +29,8 @@ constexpr int kMaxBlocks = 608;    // most blocks of k_net (4 x 152 SMs)
 constexpr int DT = 64, DR = 64;    // k_dweight: tile side, batch rows a stage
 constexpr int DLD = DT + 8;        // padded row
 constexpr int kDwThreads = 128;    // 2 x 2 warps
+constexpr int kParts = 8;          // parts below which the sums are folded,
+constexpr int kChains = 16;        // into that many chains
 
 __host__ __device__ constexpr int pad32(int d) { return (d + 31) & ~31; }
 
@@ -374,12 +376,19 @@ __device__ __forceinline__ void cp16(void *dst, const void *src, bool in) {
 // Weight gradients of every layer, dW_l[n][k] = sum over the batch of
 // dz_l[b][n] act_l[b][k]: block x takes a DT x DT tile of one layer, block y
 // `rows` rows of the batch (a multiple of DR), and writes its part to
-// parts[y].  Both operands lie batch-major; ldmatrix transposes them.  About
+// parts[y].  Both operands lie batch-major; ldmatrix transposes them.  FOLD:
+// every `chain` rows (a multiple of DR) the sums so far are added to a second
+// set and start anew, for networks with so many tiles that the batch has fewer
+// than kParts parts: the tensor core truncates its running sum at each step,
+// and over 65536 rows of two layers of 1024 units one chain left errors of
+// 4.3e-4 of the gradient, eight 4.4e-5, sixteen 1.8e-5 (ten parts, as 256 units
+// have, 2.8e-5); a training step there 2896 and 2905 us.  About
 // 450 blocks, each waiting for its operands from L2: 8.7 us for 1024 rows of
 // the 5-256-256-256-65 network, where the layers' products and column sums
 // took 36 and 59 us each.
+template <bool FOLD>
 __global__ void __launch_bounds__(kDwThreads)
-    k_dweight(const __grid_constant__ Net net, int batch, int rows) {
+    k_dweight(const __grid_constant__ Net net, int batch, int rows, int chain) {
     __shared__ __align__(16) __nv_bfloat16 sa[2][DR][DLD], sb[2][DR][DLD];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int wm = warp >> 1, wn = warp & 1;
@@ -395,6 +404,19 @@ __global__ void __launch_bounds__(kDwThreads)
     const int b0 = blockIdx.y * rows, b1 = min(batch, b0 + rows);
     const __nv_bfloat16 *A = net.dz[l], *B = net.act[l];
     float acc[2][4][4] = {};
+    float sum[2][4][4] = {};
+    int next = b0 + chain;  // row at which the sums are folded
+    auto fold = [&] {
+#pragma unroll
+        for (int mi = 0; mi < 2; ++mi)
+#pragma unroll
+            for (int ni = 0; ni < 4; ++ni)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    sum[mi][ni][q] += acc[mi][ni][q];
+                    acc[mi][ni][q] = 0.f;
+                }
+    };
     auto stage = [&](int s, int r0) {
 #pragma unroll
         for (int j = 0; j < DR * DT / 8 / kDwThreads; ++j) {
@@ -433,8 +455,15 @@ __global__ void __launch_bounds__(kDwThreads)
                     mma_bf16(acc[mi][ni], af[mi], bf[ni >> 1][(ni & 1) * 2],
                              bf[ni >> 1][(ni & 1) * 2 + 1]);
         }
+        if constexpr (FOLD) {
+            if (r0 + DR >= next) {
+                fold();
+                next += chain;
+            }
+        }
         __syncthreads();
     }
+    if constexpr (FOLD) fold();
     float *c = net.parts + blockIdx.y * net.np + net.off_w[l];
 #pragma unroll
     for (int mi = 0; mi < 2; ++mi)
@@ -444,7 +473,8 @@ __global__ void __launch_bounds__(kDwThreads)
             for (int q = 0; q < 4; ++q) {
                 const int n = n0 + wm * 32 + mi * 16 + (lane >> 2) + (q >> 1) * 8;
                 const int k = k0 + wn * 32 + ni * 8 + 2 * (lane & 3) + (q & 1);
-                if (n < N && k < K) c[(long)n * K + k] = acc[mi][ni][q];
+                if (n < N && k < K)
+                    c[(long)n * K + k] = FOLD ? sum[mi][ni][q] : acc[mi][ni][q];
             }
 }
 
@@ -654,7 +684,12 @@ cudaError_t train(lbm_mlp *h, const float *x, const float *target, int batch,
     const int stages = (batch + DR - 1) / DR;
     const int per = (stages + h->max_split - 1) / h->max_split;
     const int split = (stages + per - 1) / per;
-    k_dweight<<<dim3(h->tiles, split), kDwThreads, 0, h->stream>>>(h->net, batch, per * DR);
+    const int chain = (stages + kChains - 1) / kChains;
+    const dim3 dw(h->tiles, split);
+    if (h->max_split < kParts && per > chain)
+        k_dweight<true><<<dw, kDwThreads, 0, h->stream>>>(h->net, batch, per * DR, chain * DR);
+    else
+        k_dweight<false><<<dw, kDwThreads, 0, h->stream>>>(h->net, batch, per * DR, 0);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int nwb = (int)((h->net.np + 255) / 256), nbb = (h->net.ndb + 31) / 32;
