@@ -54,7 +54,8 @@ struct Net {
     long np;
     float *w;
     __nv_bfloat16 *wf, *wt;
-    float *hs[kMaxLayers];          // FP32 hidden activations, [batch][H]
+    float *hs[kMaxLayers];          // FP32 hidden activations of the rows that the
+                                    // blocks work on, [block][16 MT][H]
     __nv_bfloat16 *act[kMaxLayers]; // inputs of layer l in BF16
     __nv_bfloat16 *dz[kMaxLayers];  // gradients at layer l's pre-activation
     float *db;                      // [blocks of k_net][ndb]
@@ -193,6 +194,7 @@ __global__ void __launch_bounds__(32 * net_warps(MT))
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = lane >> 2, t4 = lane & 3;
     const int L = net.L;
+    const long h0 = (long)blockIdx.x * BM;  // this block's rows of hs
     __nv_bfloat16 *cur = sm, *nxt = sm + BM * ld;
     if constexpr (!TRAIN) start_after_previous();
     double lsum = 0.0;
@@ -250,7 +252,7 @@ __global__ void __launch_bounds__(32 * net_warps(MT))
                                 if (TRAIN && m < batch) {
                                     st_bf2(net.act[l + 1] + (long)m * np32 + n, v0, v1);
                                     if (n < N)
-                                        *reinterpret_cast<float2 *>(net.hs[l] + (long)m * N + n) =
+                                        *reinterpret_cast<float2 *>(net.hs[l] + (h0 + r) * N + n) =
                                             make_float2(v0, v1);
                                 }
                             } else if (!TRAIN) {
@@ -323,7 +325,7 @@ __global__ void __launch_bounds__(32 * net_warps(MT))
                                 float v0 = 0.f, v1 = 0.f;
                                 if (m < batch && n < N) {
                                     const float2 h = *reinterpret_cast<const float2 *>(
-                                        hp + (long)m * N + n);
+                                        hp + (h0 + r) * N + n);
                                     v0 = acc[mi][j][2 * hf] * (1.0f - h.x * h.x);
                                     v1 = acc[mi][j][2 * hf + 1] * (1.0f - h.y * h.y);
                                 }
@@ -780,7 +782,10 @@ lbm_status lbm_mlp_create(const lbm_mlp_shape *shape, lbm_mlp **out) {
     al(&net.wt, nt);
     const size_t zeroed = bytes;
     for (int l = 0; l <= s.n_layers; ++l) {
-        if (l < s.n_layers) al(&net.hs[l], (size_t)s.max_batch * s.n_hidden);
+        // (the blocks' rows, 64 each at most: a block is done with a tile's
+        // hidden activations before it goes on to its next tile)
+        if (l < s.n_layers)
+            al(&net.hs[l], std::min((size_t)s.max_batch, (size_t)kMaxBlocks * 64) * s.n_hidden);
         al(&net.act[l], (size_t)s.max_batch * pad32(net.dim[l]));
         al(&net.dz[l], (size_t)s.max_batch * pad32(net.dim[l + 1]));
     }
