@@ -273,13 +273,12 @@ lbm_status lbm_fit_reff(const double *t, const double *z, int32_t n,
                         double gamma, double mu, double length,
                         double cos_theta0, double *r_eff);
 
-/* Tile schedule of the TMA-staged step kernel (project addition; the paper
- * describes no implementation), computed on the host as lbm_create computes
- * it for most handles of more than 8 tiles per block (those with fewer deal
- * each block one run of consecutive tiles, and short lattices with 16 to 32
- * may have their strips evened out): the tiles of tx by ty nodes of `count`
- * lattices of nx[l] by ny[l] nodes, dealt to `grid` persistent blocks.  A strip is a run of tiles down
- * one tile column of a lattice; columns longer than
+/* Tile schedule of the TMA-staged step kernel in strips (project addition;
+ * the paper describes no implementation), computed on the host as lbm_create
+ * computes it for most handles of more than 8 tiles per block
+ * (lbm_plan_schedule has every handle's): the tiles of tx by ty nodes of
+ * `count` lattices of nx[l] by ny[l] nodes, dealt to `grid` persistent blocks.
+ * A strip is a run of tiles down one tile column of a lattice; columns longer than
  * max(4, ceil(tiles / (4 grid))) tiles are cut into strips of that length,
  * and strips go, longest first, to the block with the fewest tiles so far
  * (ties to the lower index).  Block b's k-th tile is written to
@@ -293,6 +292,17 @@ lbm_status lbm_fit_reff(const double *t, const double *z, int32_t n,
 lbm_status lbm_plan_tiles(const int32_t *nx, const int32_t *ny, int32_t count,
                           int32_t tx, int32_t ty, int32_t grid, int32_t *out,
                           int64_t cap, int32_t *slots);
+
+/* The schedule that a handle with these lattices, tiles and blocks uses, in
+ * the form of lbm_plan_tiles and with its arguments and errors: up to 8 tiles
+ * per block, each block takes one run of consecutive tiles in (lattice, tile
+ * column, row) order, their lengths one apart at most; from there on strips,
+ * those of batches with 16 to 32 tiles per block and at most 64 tiles in a
+ * column evened out (each column cut into equal pieces) where that shortens
+ * the longest list by a sixteenth.  Host-only arithmetic: needs no GPU. */
+lbm_status lbm_plan_schedule(const int32_t *nx, const int32_t *ny, int32_t count,
+                             int32_t tx, int32_t ty, int32_t grid, int32_t *out,
+                             int64_t cap, int32_t *slots);
 
 /* ---- observables without allocation ----------------------------------
  *

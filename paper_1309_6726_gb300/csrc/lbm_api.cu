@@ -1390,17 +1390,19 @@ extern "C" lbm_status lbm_load(lbm_handle *h, const char *path) {
     return LBM_OK;
 }
 
-extern "C" lbm_status lbm_plan_tiles(const int32_t *nx, const int32_t *ny,
-                                     int32_t count, int32_t tx, int32_t ty,
-                                     int32_t grid, int32_t *out, int64_t cap,
-                                     int32_t *slots) {
+// Host entry of a way of dealing tiles: checks, the schedule, its table.
+using Dealing = size_t (*)(const int32_t *, const int32_t *, int, int, int, int,
+                           std::vector<TileRec> &);
+static lbm_status export_schedule(Dealing deal, const int32_t *nx, const int32_t *ny,
+                                  int32_t count, int32_t tx, int32_t ty, int32_t grid,
+                                  int32_t *out, int64_t cap, int32_t *slots) {
     if (!nx || !ny || !slots || count < 1 || tx < 1 || ty < 1 || grid < 1)
         return fail(nullptr, LBM_EINVAL, "plan_tiles: NULL array, count, tile or grid < 1");
     for (int l = 0; l < count; ++l)
         if (nx[l] < 1 || ny[l] < 1)
             return fail(nullptr, LBM_EINVAL, "plan_tiles: lattice size < 1");
     std::vector<TileRec> sched;
-    const size_t n = plan_tiles(nx, ny, count, tx, ty, grid, sched);
+    const size_t n = deal(nx, ny, count, tx, ty, grid, sched);
     *slots = (int32_t)n;
     if (!out) return LBM_OK;
     if ((int64_t)sched.size() * 3 > cap)
@@ -1411,6 +1413,20 @@ extern "C" lbm_status lbm_plan_tiles(const int32_t *nx, const int32_t *ny,
         out[3 * k + 2] = sched[k].lat >= 0 ? sched[k].y0 : 0;
     }
     return LBM_OK;
+}
+
+extern "C" lbm_status lbm_plan_tiles(const int32_t *nx, const int32_t *ny,
+                                     int32_t count, int32_t tx, int32_t ty,
+                                     int32_t grid, int32_t *out, int64_t cap,
+                                     int32_t *slots) {
+    return export_schedule(plan_tiles, nx, ny, count, tx, ty, grid, out, cap, slots);
+}
+
+extern "C" lbm_status lbm_plan_schedule(const int32_t *nx, const int32_t *ny,
+                                        int32_t count, int32_t tx, int32_t ty,
+                                        int32_t grid, int32_t *out, int64_t cap,
+                                        int32_t *slots) {
+    return export_schedule(deal_tiles, nx, ny, count, tx, ty, grid, out, cap, slots);
 }
 
 extern "C" lbm_status lbm_fit_reff(const double *t, const double *z,

@@ -26,7 +26,7 @@ SYMBOLS = ("lbm_create", "lbm_create_batch", "lbm_set_stream", "lbm_step",
            "lbm_set_fields",
            "lbm_save", "lbm_load", "lbm_destroy", "lbm_last_error",
            "lbm_fit_reff", "lbm_observables_static", "lbm_autotune",
-           "lbm_get_tuning", "lbm_plan_tiles")
+           "lbm_get_tuning", "lbm_plan_tiles", "lbm_plan_schedule")
 
 
 class LbmError(RuntimeError):
@@ -127,6 +127,7 @@ def load_library(path: str = LIB_PATH):
     ip = C.POINTER(C.c_int32)
     lib.lbm_plan_tiles.argtypes = [ip, ip, C.c_int32, C.c_int32, C.c_int32,
                                    C.c_int32, ip, C.c_int64, ip]
+    lib.lbm_plan_schedule.argtypes = lib.lbm_plan_tiles.argtypes
     lib.lbm_autotune.argtypes = [vp, C.c_int32, C.POINTER(Tuning)]
     lib.lbm_get_tuning.argtypes = [vp, C.POINTER(Tuning)]
     lib.lbm_observables_static.argtypes = [vp, vp, vp, vp, C.c_int32,
@@ -381,26 +382,36 @@ def fit_reff(t, z, gamma: float, mu: float, length: float,
     return out.value
 
 
-def plan_tiles(sizes, tx: int, ty: int, grid: int) -> np.ndarray:
-    """Tile schedule of the TMA step kernel (``lbm_plan_tiles``) for
-    lattices of (nx, ny) ``sizes``: int32 [slots, grid, 3] of (lattice,
-    first column, first row), lattice -1 after a block's last tile."""
+def _schedule(entry: str, sizes, tx: int, ty: int, grid: int) -> np.ndarray:
     lib = load_library()
+    call = getattr(lib, entry)
     nx = np.ascontiguousarray([s[0] for s in sizes], dtype=np.int32)
     ny = np.ascontiguousarray([s[1] for s in sizes], dtype=np.int32)
     ip = C.POINTER(C.c_int32)
     slots = C.c_int32()
     args = (nx.ctypes.data_as(ip), ny.ctypes.data_as(ip), len(nx), tx, ty,
             grid)
-    st = lib.lbm_plan_tiles(*args, None, 0, C.byref(slots))
+    st = call(*args, None, 0, C.byref(slots))
     if st != LBM_OK:
         raise LbmError(st, lib.lbm_last_error(None).decode())
     out = np.empty((slots.value, grid, 3), dtype=np.int32)
-    st = lib.lbm_plan_tiles(*args, out.ctypes.data_as(ip), out.size,
-                            C.byref(slots))
+    st = call(*args, out.ctypes.data_as(ip), out.size, C.byref(slots))
     if st != LBM_OK:
         raise LbmError(st, lib.lbm_last_error(None).decode())
     return out
+
+
+def plan_tiles(sizes, tx: int, ty: int, grid: int) -> np.ndarray:
+    """Tile schedule in strips (``lbm_plan_tiles``) for lattices of (nx, ny)
+    ``sizes``: int32 [slots, grid, 3] of (lattice, first column, first row),
+    lattice -1 after a block's last tile."""
+    return _schedule("lbm_plan_tiles", sizes, tx, ty, grid)
+
+
+def plan_schedule(sizes, tx: int, ty: int, grid: int) -> np.ndarray:
+    """The schedule that a handle uses (``lbm_plan_schedule``), in the form
+    of :func:`plan_tiles`."""
+    return _schedule("lbm_plan_schedule", sizes, tx, ty, grid)
 
 
 #: most columns lbm_observables_static accepts (its fixed scratch size)
