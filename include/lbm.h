@@ -258,6 +258,12 @@ lbm_status lbm_autotune(lbm_handle *h, int32_t steps, lbm_tuning *out);
 /* The variant in use. */
 lbm_status lbm_get_tuning(const lbm_handle *h, lbm_tuning *out);
 
+/* Whether longer calls keep this handle's state on chip (see lbm_step): the
+ * blocks per cluster, one cluster per lattice, with the nodes of a block's
+ * tile in *tx and *ty (each may be NULL); 0, and nothing written, where every
+ * step is a launch; -1 for a NULL handle. */
+int32_t lbm_get_on_chip(const lbm_handle *h, int32_t *tx, int32_t *ty);
+
 /* Frees everything; NULL is allowed. */
 void lbm_destroy(lbm_handle *h);
 

@@ -1460,6 +1460,15 @@ extern "C" lbm_status lbm_get_tuning(const lbm_handle *h, lbm_tuning *out) {
     return LBM_OK;
 }
 
+extern "C" int32_t lbm_get_on_chip(const lbm_handle *h, int32_t *tx, int32_t *ty) {
+    if (!h) return -1;
+    if (h->csize > 0) {
+        if (tx) *tx = h->ctx;
+        if (ty) *ty = h->cty;
+    }
+    return h->csize;
+}
+
 extern "C" lbm_status lbm_autotune(lbm_handle *h, int32_t steps,
                                    lbm_tuning *out) {
     if (!h || steps < 1) return fail(h, LBM_EINVAL, "bad handle or steps < 1");

@@ -26,7 +26,7 @@ SYMBOLS = ("lbm_create", "lbm_create_batch", "lbm_set_stream", "lbm_step",
            "lbm_set_fields",
            "lbm_save", "lbm_load", "lbm_destroy", "lbm_last_error",
            "lbm_fit_reff", "lbm_observables_static", "lbm_autotune",
-           "lbm_get_tuning", "lbm_plan_tiles", "lbm_plan_schedule")
+           "lbm_get_tuning", "lbm_get_on_chip", "lbm_plan_tiles", "lbm_plan_schedule")
 
 
 class LbmError(RuntimeError):
@@ -130,6 +130,8 @@ def load_library(path: str = LIB_PATH):
     lib.lbm_plan_schedule.argtypes = lib.lbm_plan_tiles.argtypes
     lib.lbm_autotune.argtypes = [vp, C.c_int32, C.POINTER(Tuning)]
     lib.lbm_get_tuning.argtypes = [vp, C.POINTER(Tuning)]
+    lib.lbm_get_on_chip.argtypes = [vp, ip, ip]
+    lib.lbm_get_on_chip.restype = C.c_int32
     lib.lbm_observables_static.argtypes = [vp, vp, vp, vp, C.c_int32,
                                            C.c_int32, C.c_int32, C.c_int32,
                                            dp, C.c_int64, C.c_int64, vp, vp]
@@ -359,6 +361,13 @@ class Solver:
         t = Tuning()
         self._check(self._lib.lbm_get_tuning(self._h, C.byref(t)))
         return t.as_dict()
+
+    def on_chip(self):
+        """(tile, blocks per cluster) of the steps that longer calls keep on
+        chip, e.g. ("32x4", 8); None where every step is a launch."""
+        tx, ty = C.c_int32(), C.c_int32()
+        n = self._lib.lbm_get_on_chip(self._h, C.byref(tx), C.byref(ty))
+        return ("%dx%d" % (tx.value, ty.value), n) if n > 0 else None
 
     def save(self, path: str) -> None:
         self._check(self._lib.lbm_save(self._h, path.encode()))
