@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -491,6 +492,11 @@ static size_t lay_strips(const std::vector<Strip> &strips, int tx, int ty, int g
     return slots;
 }
 
+// Most tiles of a strip of plan_tiles.
+static long long strip_rows(long long total, int grid) {
+    return std::max(4LL, (total + 4LL * grid - 1) / (4LL * grid));
+}
+
 // Tile schedule of the persistent TMA kernel, host arithmetic only.  A
 // strip is a run of tiles down one tile column of a lattice (the halo rows
 // each tile copies were just copied by the tile above it).  Columns taller
@@ -505,8 +511,7 @@ static size_t plan_tiles(const int32_t *nx, const int32_t *ny, int count,
     long long total = 0;
     for (int l = 0; l < count; ++l)
         total += (long long)((nx[l] + tx - 1) / tx) * ((ny[l] + ty - 1) / ty);
-    const long long seg =
-        std::max(4LL, (total + 4LL * grid - 1) / (4LL * grid));
+    const long long seg = strip_rows(total, grid);
     std::vector<Strip> strips;
     for (int l = 0; l < count; ++l) {
         const int cols = (nx[l] + tx - 1) / tx, rows = (ny[l] + ty - 1) / ty;
@@ -545,36 +550,60 @@ constexpr int kRunTiles = 8;  // most tiles per block dealt as runs
 // gives (1024 x 1024 preform BF16 42.5 / 44.5).
 constexpr int kEvenFrom = 16, kEvenTo = 32, kEvenRows = 64;
 
-// As plan_tiles, but each tile column is cut into equal pieces (their lengths
-// differ by one), of the length 3 to 8 that leaves the fullest block the
-// least, the longest such.
+// Tiles of the fullest block when strips, `by_rows` of each length, are dealt
+// as deal_strips deals them: which of the emptiest blocks takes a strip makes
+// no difference to the loads, so blocks and strips are counted, not listed.
+static long long fullest_block(const std::map<int, long long> &by_rows, int grid) {
+    std::map<long long, long long> blocks{{0, grid}};  // blocks of each load
+    for (auto r = by_rows.rbegin(); r != by_rows.rend(); ++r)
+        for (long long left = r->second; left > 0;) {
+            const auto low = blocks.begin();
+            const long long load = low->first, n = std::min(left, low->second);
+            if ((low->second -= n) == 0) blocks.erase(low);
+            blocks[load + r->first] += n;
+            left -= n;
+        }
+    return blocks.rbegin()->first;
+}
+
+// Strips as plan_tiles, but each tile column cut into equal pieces (their
+// lengths differ by one), of the length 3 to 8 that leaves the fullest block
+// the least, the longest such.  Returns the slots per block, or 0 where that
+// is not a sixteenth below `plain`; the strips are listed and dealt once, when
+// it is known that they are taken.
 static size_t even_strips(const int32_t *nx, const int32_t *ny, int count, int tx,
-                          int ty, int grid, std::vector<TileRec> &sched) {
-    std::vector<Strip> strips, best;
-    std::vector<std::vector<int>> lists, best_lists;
-    std::vector<long long> load, best_load;
-    long long best_max = 0;
-    for (int seg = 8; seg >= 3; --seg) {
-        strips.clear();
+                          int ty, int grid, long long plain, std::vector<TileRec> &sched) {
+    long long top = 0;
+    int seg = 0;
+    for (int len = 8; len >= 3; --len) {
+        std::map<int, long long> by_rows;
         for (int l = 0; l < count; ++l) {
             const int cols = (nx[l] + tx - 1) / tx, rows = (ny[l] + ty - 1) / ty;
-            const int n = (rows + seg - 1) / seg;
-            for (int c = 0; c < cols; ++c)
-                for (int k = 0; k < n; ++k) {
-                    const int r0 = (int)((long long)k * rows / n);
-                    strips.push_back({l, c, r0, (int)((long long)(k + 1) * rows / n) - r0});
-                }
+            const int n = (rows + len - 1) / len;
+            by_rows[rows / n] += (long long)cols * (n - rows % n);
+            if (rows % n) by_rows[rows / n + 1] += (long long)cols * (rows % n);
         }
-        deal_strips(strips, grid, lists, load);
-        const long long top = *std::max_element(load.begin(), load.end());
-        if (best.empty() || top < best_max) {
-            best_max = top;
-            best = strips;
-            best_lists = lists;
-            best_load = load;
+        const long long t = fullest_block(by_rows, grid);
+        if (seg == 0 || t < top) {
+            top = t;
+            seg = len;
         }
     }
-    return lay_strips(best, tx, ty, grid, best_lists, best_load, sched);
+    if (16 * top > 15 * plain) return 0;
+    std::vector<Strip> strips;
+    for (int l = 0; l < count; ++l) {
+        const int cols = (nx[l] + tx - 1) / tx, rows = (ny[l] + ty - 1) / ty;
+        const int n = (rows + seg - 1) / seg;
+        for (int c = 0; c < cols; ++c)
+            for (int k = 0; k < n; ++k) {
+                const int r0 = (int)((long long)k * rows / n);
+                strips.push_back({l, c, r0, (int)((long long)(k + 1) * rows / n) - r0});
+            }
+    }
+    std::vector<std::vector<int>> lists;
+    std::vector<long long> load;
+    deal_strips(strips, grid, lists, load);
+    return lay_strips(strips, tx, ty, grid, lists, load, sched);
 }
 
 static size_t deal_tiles(const int32_t *nx, const int32_t *ny, int count,
@@ -583,19 +612,22 @@ static size_t deal_tiles(const int32_t *nx, const int32_t *ny, int count,
     for (int l = 0; l < count; ++l)
         total += (long long)((nx[l] + tx - 1) / tx) * ((ny[l] + ty - 1) / ty);
     if (total > (long long)kRunTiles * grid) {
-        const size_t slots = plan_tiles(nx, ny, count, tx, ty, grid, sched);
         int tall = 0;
         for (int l = 0; l < count; ++l) tall = std::max(tall, (ny[l] + ty - 1) / ty);
         if (total > (long long)kEvenFrom * grid && total <= (long long)kEvenTo * grid &&
             tall <= kEvenRows) {
-            std::vector<TileRec> even;
-            const size_t n = even_strips(nx, ny, count, tx, ty, grid, even);
-            if (16 * n <= 15 * slots) {
-                sched.swap(even);
-                return n;
+            const int seg = (int)strip_rows(total, grid);
+            std::map<int, long long> by_rows;
+            for (int l = 0; l < count; ++l) {
+                const int cols = (nx[l] + tx - 1) / tx, rows = (ny[l] + ty - 1) / ty;
+                if (rows / seg) by_rows[seg] += (long long)cols * (rows / seg);
+                if (rows % seg) by_rows[rows % seg] += cols;
             }
+            const size_t n = even_strips(nx, ny, count, tx, ty, grid,
+                                         fullest_block(by_rows, grid), sched);
+            if (n > 0) return n;
         }
-        return slots;
+        return plan_tiles(nx, ny, count, tx, ty, grid, sched);
     }
     const size_t slots = (size_t)((total + grid - 1) / grid);
     sched.assign((size_t)grid * slots, TileRec{-1, 0, 0, 0});

@@ -110,6 +110,26 @@ def test_random_batches():
     assert kinds == {"runs", "strips", "evened"}
 
 
+@pytest.mark.parametrize("count", [4, 5, 8, 10])
+def test_evened_strips_cost_no_more_than_a_few_plain_ones(count):
+    # a handle's schedule is part of every create: choosing among six lengths
+    # must not deal the batch six times (measured 6 to 8 times plan_tiles then)
+    import time
+    from paper_1309_6726_gb300 import inputs as I
+    sizes = [(m.length + 96, m.width + 2) for m in I.sweep_members(512)[:count]]
+
+    def fastest(f):
+        best = math.inf
+        for _ in range(40):
+            t = time.perf_counter()
+            f(sizes, 64, 4, 304)
+            best = min(best, time.perf_counter() - t)
+        return best
+    ratio = fastest(lbm.plan_schedule) / fastest(lbm.plan_tiles)
+    print("%d lattices: %.2f" % (count, ratio))
+    assert ratio < 3
+
+
 def test_rejects_what_plan_tiles_rejects():
     for args in (([], 64, 8, 152), ([(64, 8)], 0, 8, 152), ([(64, 8)], 64, 8, 0),
                  ([(0, 8)], 64, 8, 4)):
