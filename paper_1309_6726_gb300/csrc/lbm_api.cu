@@ -275,19 +275,41 @@ static bool reads_pageable() {
     return on != 0;
 }
 
-// Share of solid nodes, from every 16th row; 0 where the host cannot read the
-// array.
-static double solid_share(const lbm_geometry &g) {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, g.solid) != cudaSuccess) {
-        cudaGetLastError();
-        return 0.0;
+// Share of solid nodes inside the lattices of a batch of `nodes` nodes, from
+// evenly spaced rows, about 64k nodes in all (the outermost rows, walls of a
+// capillary, are left out).  Device arrays: one strided copy for each of 32
+// lattices at most.
+static double solid_share(const lbm_geometry *g, int count, int64_t nodes) {
+    const int64_t step = std::max<int64_t>(16, nodes >> 16);
+    int64_t solid = 0, seen = 0, copies = 0;
+    std::vector<uint8_t> rows;
+    for (int l = 0; l < count; ++l) {
+        const int64_t nx = g[l].nx, ny = g[l].ny, y0 = std::min(step, ny) / 2;
+        const int64_t n = (ny - 2 - y0) / step + 1;  // rows y0, y0 + step, ... < ny - 1
+        const uint8_t *src = g[l].solid + y0 * nx;
+        int64_t pitch = step * nx;
+        cudaPointerAttributes a;
+        if (cudaPointerGetAttributes(&a, src) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        if (a.type == cudaMemoryTypeDevice) {
+            if (l * 32LL / count < copies) continue;
+            ++copies;
+            rows.resize(n * nx);
+            if (cudaMemcpy2D(rows.data(), nx, src, pitch, nx, n, cudaMemcpyDeviceToHost) !=
+                cudaSuccess) {
+                cudaGetLastError();
+                continue;
+            }
+            src = rows.data();
+            pitch = nx;
+        }
+        for (int64_t r = 0; r < n; ++r)
+            for (int64_t x = 0; x < nx; ++x) solid += src[r * pitch + x] != 0;
+        seen += n * nx;
     }
-    if (a.type == cudaMemoryTypeDevice) return 0.0;
-    int64_t n = 0, rows = 0;
-    for (int64_t y = 0; y < g.ny; y += 16, ++rows)
-        for (int64_t x = 0; x < g.nx; ++x) n += g.solid[y * g.nx + x] != 0;
-    return (double)n / (double)(rows * g.nx);
+    return seen > 0 ? (double)solid / (double)seen : 0.0;
 }
 
 static void pick_tile(lbm_handle *h, const lbm_geometry *g) {
@@ -301,6 +323,18 @@ static void pick_tile(lbm_handle *h, const lbm_geometry *g) {
     // 2048 x 2048 box 137 / 154, preform 142 / 242).
     constexpr int kSms = 152;
     constexpr int64_t kLargeLattice = 640000, kLargeBatch = 24000000;
+    // FP32 batches with solid nodes inside, of more than L2 holds of both
+    // buffers (1.2M nodes, 210 MB): 64 x 8 too.  64 x 4 stores node by node,
+    // and rows with solid nodes leave holes in the sectors on their way to
+    // memory; the more of them turn solid, the more it loses.  64 x 8 / 64 x 4:
+    // 16 preforms of 512 x 512, 5 % solid 147 / 165, 25 % 150 / 207; random
+    // solid nodes, 24 of 512 x 512, 3 % 290 / 311, and when growth has filled
+    // half 227 / 346; 15 % 306 / 382; four of 4096 x 128, 3 % 101 / 101 and 79 /
+    // 105; two of 790 x 800 (1.26M), 3 % 72.0 / 69.4 and 58.8 / 69.6.  At 1 %
+    // 64 x 4 is ahead (24 of 512 x 512 269 / 251), as in smaller batches (four
+    // preforms of 512 x 512 44.9 / 41.2, one of 790 x 800 45.2 / 42.6).
+    constexpr int64_t kSolidBatch = 1200000;
+    constexpr double kSolidInside = 0.02;
     int64_t small = 0, nodes = 0, most = 0;
     for (int l = 0; l < h->count; ++l) {
         const int64_t n = (int64_t)g[l].nx * g[l].ny;
@@ -309,7 +343,12 @@ static void pick_tile(lbm_handle *h, const lbm_geometry *g) {
         most = std::max(most, n);
     }
     h->tx = 64;
-    h->ty = !h->half && (most > kLargeLattice || nodes > kLargeBatch) ? 8 : 4;
+    h->ty = 4;
+    if (!h->half &&
+        (most > kLargeLattice || nodes > kLargeBatch ||
+         (h->count > 1 && nodes > kSolidBatch &&
+          solid_share(g, h->count, nodes) >= kSolidInside)))
+        h->ty = 8;
     // Where 32 x 4 tiles leave no SM more than one tile, a step is one tile's
     // latency, which the smaller block shortens: 256 x 32 (64 tiles) 64 x 4 /
     // 32 x 4: FP32 5.5 / 4.3, FP16 5.3 / 4.5; beyond (1000 x 60, 480 tiles)
@@ -321,7 +360,8 @@ static void pick_tile(lbm_handle *h, const lbm_geometry *g) {
     // One FP32 lattice of that size up to 1.5M nodes, a quarter or more of it
     // solid: 32 x 8 (preform, 64 x 8 / 32 x 8: 1024 x 1024 44.8 / 40.6, 1448 x
     // 1448 75.4 / 80.5, 2048 x 2048 142 / 170).
-    if (h->ty == 8 && h->count == 1 && nodes <= 1500000 && solid_share(g[0]) >= 0.25)
+    if (h->ty == 8 && h->count == 1 && nodes <= 1500000 &&
+        solid_share(g, 1, nodes) >= 0.25)
         h->tx = 32;
     const char *e = getenv("LBM_TILE");
     if (e) {
