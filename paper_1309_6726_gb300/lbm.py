@@ -6,6 +6,7 @@ CUDA device is missing, constructing a :class:`Solver` raises.
 from __future__ import annotations
 
 import ctypes as C
+import mmap
 import os
 
 import numpy as np
@@ -156,11 +157,15 @@ def _params(p, precision: int) -> Params:
 
 
 def _fresh(shape, dtype) -> np.ndarray:
-    """An array for a read-back, its pages present: the device's copy into
-    pages that the host has not touched yet faults on each of them (up to 12
-    ms for 12.6 MB instead of 0.11; touching them first 0.035)."""
+    """An array for a read-back (which writes all of it).  Of more than 64 KB
+    and up to 32 MB, where malloc recycles memory, its pages are made present
+    first: the device's copy into pages that the host has not touched yet
+    faults on each of them (up to 12 ms for 12.6 MB instead of 0.11).  Above
+    32 MB every page is new, and the copy takes the faults faster than the
+    host does (370 MB 15.7 ms, touched first 16.9)."""
     out = np.empty(shape, dtype)
-    out.reshape(-1).view(np.uint8)[::4096] = 0
+    if 1 << 16 < out.nbytes <= 32 << 20:
+        out.reshape(-1).view(np.uint8)[::mmap.PAGESIZE] = 0
     return out
 
 
@@ -297,7 +302,7 @@ class Solver:
         runs at the link's full rate)."""
         sizes = [ny * nx for ny, nx in self.shapes]
         if out is None:
-            buf = _fresh(sum(sizes), np.uint8)
+            buf = _fresh((sum(sizes),), np.uint8)
         else:
             buf = out.reshape(-1)
             if (buf.dtype != np.uint8 or buf.size != sum(sizes)
