@@ -747,9 +747,9 @@ static lbm_status retile(lbm_handle *h, bool tma, int tx, int ty) {
         d.tile_base = tiles;
         tiles += d.tiles_x * ((d.ny + ty - 1) / ty);
     }
+    CK(h, cudaMemcpyAsync(h->d_desc, h->desc.data(), h->count * sizeof(LatDesc),
+                          cudaMemcpyHostToDevice, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
-    CK(h, cudaMemcpy(h->d_desc, h->desc.data(), h->count * sizeof(LatDesc),
-                     cudaMemcpyHostToDevice));
     h->ntiles = tiles;
     if (h->d_sched) cudaFree(h->d_sched);
     h->d_sched = nullptr;
@@ -1451,7 +1451,12 @@ extern "C" lbm_status lbm_load(lbm_handle *h, const char *path) {
         while (ok && done < bytes) {
             const size_t n = std::min(buf.size(), bytes - done);
             ok = fread(buf.data(), 1, n, f) == n;
-            if (ok && cudaMemcpy((uint8_t *)dptr + done, buf.data(), n, cudaMemcpyHostToDevice) != cudaSuccess)
+            // on the handle's stream: a plain copy from pageable memory may
+            // return before it has landed, and nothing orders the handle's
+            // next launch behind it
+            if (ok && (cudaMemcpyAsync((uint8_t *)dptr + done, buf.data(), n,
+                                       cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
+                       cudaStreamSynchronize(h->stream) != cudaSuccess))
                 ok = false;
             done += n;
         }

@@ -69,3 +69,27 @@ def test_load_refuses_other_parameters(tmp_path):
     with lbm.Solver(I.random_lattice(296, 40, seed=1), MP) as b, \
             pytest.raises(lbm.LbmError):
         b.load(path)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+def test_steps_queued_right_after_a_load(precision, tmp_path):
+    # nothing but the stream's order stands between the upload and the steps
+    # (the step counter is the last thing uploaded), with other work around
+    import torch
+    from paper_1309_6726_gb300 import lbm
+    g = I.random_lattice(300, 40, seed=1)
+    path = str(tmp_path / "state")
+    x = torch.ones(1 << 24, device="cuda")
+    with lbm.Solver(g, MP, precision) as a, lbm.Solver(g, MP, precision) as b:
+        a.step(17)
+        a.save(path)
+        a.step(9)
+        want, mask = a.populations(), a.solid_mask()
+        for _ in range(10):
+            b.step(3)
+            x.add_(1.0)
+            b.load(path)
+            b.step(9)
+            assert b.observables_array(allow_nan=True)["step"][0] == 26
+            np.testing.assert_array_equal(b.populations(), want)
+            np.testing.assert_array_equal(b.solid_mask(), mask)
