@@ -25,7 +25,7 @@ def test_schedules_give_the_same_steps(sizes, kind, precision, monkeypatch):
     even = not np.array_equal(lbm.plan_schedule(sizes, 64, 4, grid),
                               lbm.plan_tiles(sizes, 64, 4, grid))
     assert kind == ("runs" if tiles <= 8 * grid else "evened" if even else "strips")
-    geoms = [I.random_lattice(nx, ny, seed=k, solid_fraction=0.02)
+    geoms = [I.random_lattice(nx, ny, seed=k, solid_fraction=0.01)
              for k, (nx, ny) in enumerate(sizes)]
     mps = [I.ModelParams(g_ads=0.3, k_r=1e-2, m_threshold=0.05, inlet=1)] * len(sizes)
     got = []
