@@ -758,6 +758,7 @@ static lbm_status retile(lbm_handle *h, bool tma, int tx, int ty) {
         std::vector<CUtensorMap> maps;
         std::vector<TileRec> sched;
         if (!make_maps(h, maps, why) || !make_schedule(h, sched, why)) {
+            cudaStreamSynchronize(h->stream);  // (what was issued reads the vectors)
             cudaGetLastError();
             return fail(h, LBM_EINVAL, "tile shape not supported: " + why);
         }
