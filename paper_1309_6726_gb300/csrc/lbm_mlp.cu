@@ -599,6 +599,7 @@ struct lbm_mlp {
     int max_split = 1;   // parts of the weight gradients
     cudaStream_t own = nullptr, stream = nullptr;
     cudaEvent_t moved = nullptr;  // end of the work queued before a change of stream
+    bool queued = false;          // the stream holds work that no call waited for
     long adam_t = 0;
     std::string err;
     bool dead = false;
@@ -657,6 +658,7 @@ int pick_mt(const lbm_mlp *h, int batch, bool train) {
 template <bool TRAIN>
 cudaError_t launch_net(lbm_mlp *h, const float *x, const float *target, int batch,
                        float *y, float inv_count, int *blocks) {
+    h->queued = true;
     const int mt = pick_mt(h, batch, TRAIN);
     const int grid = std::min((batch + 16 * mt - 1) / (16 * mt), kMaxBlocks);
     const size_t sm = net_smem(h, mt);
@@ -731,6 +733,7 @@ lbm_status read_loss(lbm_mlp *h, double *loss) {
     MCK(h, cudaMemcpyAsync(loss, h->d_loss, sizeof(double),
                            cudaMemcpyDeviceToHost, h->stream));
     MCK(h, cudaStreamSynchronize(h->stream));
+    h->queued = false;
     return LBM_OK;
 }
 }  // namespace
@@ -839,6 +842,7 @@ lbm_status lbm_mlp_set_params(lbm_mlp *h, const float *host, int64_t n) {
     MCK(h, cudaGetLastError());
     // the host array may be reused as soon as this returns
     MCK(h, cudaStreamSynchronize(h->stream));
+    h->queued = false;
     h->adam_t = 0;
     return LBM_OK;
 }
@@ -850,6 +854,7 @@ lbm_status lbm_mlp_get_params(lbm_mlp *h, float *host, int64_t n) {
     MCK(h, cudaMemcpyAsync(host, h->net.w, n * sizeof(float), cudaMemcpyDeviceToHost,
                            h->stream));
     MCK(h, cudaStreamSynchronize(h->stream));
+    h->queued = false;
     return LBM_OK;
 }
 
@@ -862,7 +867,7 @@ lbm_status lbm_mlp_set_stream(lbm_mlp *h, void *cuda_stream) {
     // (A stream that is being captured can neither wait for work outside the
     // capture nor be waited for from outside: there the caller orders the
     // replays, as with any captured work.)
-    if (!h->dead && !capturing(h->stream) && !capturing(to)) {
+    if (h->queued && !h->dead && !capturing(h->stream) && !capturing(to)) {
         MCK(h, cudaEventRecord(h->moved, h->stream));
         MCK(h, cudaStreamWaitEvent(to, h->moved, 0));
     }
