@@ -1,8 +1,8 @@
 // lbm_api.cu -- the C ABI declared in include/lbm.h: handle life cycle,
 // packed ragged layout of a batch, stepping, observables, field access,
 // checkpoints.  All arithmetic of the method runs in the kernels of
-// lbm_step.cu and lbm_aux.cu; this file only sizes, allocates, copies and
-// launches.
+// lbm_step_tma.cu, lbm_step_cluster.cu, lbm_step.cu and lbm_aux.cu; this file
+// sizes, allocates, copies, deals the tiles and launches.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -316,11 +316,15 @@ static void pick_tile(lbm_handle *h, const lbm_geometry *g) {
     // Measured, us per step.  FP16: 64 x 4, two 256-thread blocks per SM, on
     // every workload (sweep of 40 lattices 248 at 64 x 8, 241 at 64 x 4).
     // FP32: the same where it wins, in lattices up to 640k nodes of batches up
-    // to 24M (64 x 8 / 64 x 4: 4096 x 128 22.4 / 19.8, sweep of 40 lattices
-    // 254 / 247, of 96 627 / 620); its stores go to 22 planes at once, and in
+    // to 24M (64 x 8 / 64 x 4: 4096 x 128 20.8 / 18.7, sweep of 40 lattices
+    // 252 / 244, of 100 644 / 638); its stores go to 22 planes at once, and in
     // larger planes or batches one 512-thread block of 64 x 8 with an output
     // tile is ahead (sweep of 192 lattices 1175 / 1270, of 512 3118 / 3521;
-    // 2048 x 2048 box 137 / 154, preform 142 / 242).
+    // 2048 x 2048 box 137 / 154, preform 142 / 242).  640k nodes: both buffers
+    // take 113 MB, about what L2 holds; beyond, the stores reach memory.  24M:
+    // the line lies between the sweeps of 100 lattices (20M) and of 192 (38M);
+    // what turns there was not isolated.  (Solid-free boxes of 6M nodes in
+    // batches are past it already: 24 of 512 x 512 220 / 235.)
     constexpr int kSms = 152;
     constexpr int64_t kLargeLattice = 640000, kLargeBatch = 24000000;
     // FP32 batches with solid nodes inside, of more than L2 holds of both

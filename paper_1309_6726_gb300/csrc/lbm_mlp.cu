@@ -22,8 +22,8 @@ namespace lbmmlp {
 
 constexpr int kMaxLayers = 9;      // L hidden + output
 // warps of a k_net block, side by side along the units: 16 for 16 rows, where
-// latency is all there is (8 -> 16: 256 rows forward 10.5 -> 9.1 us, a
-// training step on 1024 rows 38.3 -> 32.6), else 8
+// latency is all there is (8 -> 16: 256 rows forward 10.1 -> 8.6 us, a
+// training step on 1024 rows 36.9 -> 32.6), else 8
 __host__ __device__ constexpr int net_warps(int mt) { return mt == 1 ? 16 : 8; }
 constexpr int kMaxBlocks = 608;    // most blocks of k_net (4 x 152 SMs)
 constexpr int DT = 64, DR = 64;    // k_dweight: tile side, batch rows a stage
@@ -97,7 +97,8 @@ __device__ __forceinline__ void st_bf2(__nv_bfloat16 *p, float a, float b) {
 // Programmatic dependent launch of the inference pass: its blocks start under
 // the tail of the launch before it in the stream, let the next one start at
 // once and wait here for the previous launch to end before they touch memory
-// (256 rows forward, back to back 10.5 -> 9.0 us, 8192 rows 20.6 -> 19.0).
+// (back to back: 256 rows forward 8.7 -> 8.6 us, 1024 rows 9.1 -> 8.7, 8192
+// rows 18.9 -> 18.5).
 // Training's three launches are plain: with the weight gradients' blocks
 // waiting on the SMs a step on 8192 rows took 102 us instead of 89.
 __device__ __forceinline__ void start_after_previous() {
@@ -181,7 +182,7 @@ struct Product {
 // Bound by latency: the chain of products, each with 128 KB of weights from L2
 // per block, and the epilogues' tanh (tensor pipe 4 % busy in training on 1024
 // rows, 23 % forward on 8192).  One launch per product took 133 us forward on
-// 256 rows and 158 on 8192; this 9.1 and 19.0.
+// 256 rows and 158 on 8192; this 8.6 and 18.5.
 template <int MT, bool TRAIN>
 __global__ void __launch_bounds__(32 * net_warps(MT))
     k_net(const __grid_constant__ Net net, const float *__restrict__ x,

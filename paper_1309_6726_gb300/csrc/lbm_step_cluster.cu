@@ -11,12 +11,14 @@
 // flags.  Per node the step is that of lbm_step_tma.cu, in the same order, so
 // the results are the same bit for bit.
 //
-// What bounds it: the latency of one tile's step -- pull and density ring
-// about 1300 cycles, update 1100 to 2000, the stores to other blocks and the
-// cluster barrier 2500 (256 x 32, FP32, 64 x 8 tiles).  Against one launch per
-// step (which adds the launch, the reload from L2 and the drain of the
-// stores): 256 x 32 FP32 3.9 -> 2.9 us per step, FP16 3.9 -> 3.2, 131 x 13
-// FP16 3.8 -> 3.3.  Stores to other blocks are what the halo costs: sending
+// What bounds it: the latency of one tile's step.  Stamped per warp (256 x 32,
+// FP32, 64 x 8 tiles): pull and density ring 960 cycles (1580 in the warps that
+// take the ring), update with the stores to other blocks 3090, cluster barrier
+// 1270 to arrive (its release waits for those stores) and 860 to pass; issue
+// slots 38 % busy, top stalls barrier 1.9 and membar 1.5 per issue.  Against
+// one launch per step (which adds the launch, the reload from L2 and the drain
+// of the stores): 256 x 32 FP32 3.9 -> 2.7 us per step, FP16 3.9 -> 3.05, 131 x
+// 13 FP16 3.8 -> 3.3.  Stores to other blocks are what the halo costs: sending
 // every value of the two edge rows and columns, from the registers or copied
 // from shared memory afterwards in 16-byte words, measured 3.3 and 3.5 us;
 // only what the other tile reads goes out.

@@ -14,8 +14,9 @@
 //     one is computed;
 //   * all pulls -- the tile's own nodes and the one-node density ring the
 //     cohesion stencil needs -- then read shared memory at fixed offsets;
-//   * the tile's post-collision values go to a shared output tile that one
-//     bulk tensor store per tile copies out;
+//   * the post-collision values of tiles up to 256 nodes are stored node by
+//     node; larger tiles, and FP32 32 x 8, write them to a shared output tile
+//     that one bulk tensor store copies out (TmaTile::NOUT);
 //   * the lattice planes carry a two-node periodic ghost band (rows and
 //     columns), so every copy reads valid neighbours and nothing needs
 //     patching;
