@@ -187,10 +187,11 @@ lbm_status lbm_set_stream(lbm_handle *h, void *cuda_stream);
  * rho_B and C over the nodes it updates), which the next lbm_observables
  * then reads instead of every node's populations.
  * While the caller captures the bound stream, a call of fewer than 16 steps is
- * captured as launches (longer ones are refused).  They read the buffer that is
- * current then: with an even number of steps, replays continue from the state
- * whenever the steps taken by other calls in between are even in all.  The
- * step count of the handle counts the captured call, not its replays. */
+ * captured as launches (longer ones fail, and end the handle).  These read the
+ * buffer that is current then: with an even number of steps, replays continue
+ * from the state whenever the steps taken by other calls in between are even
+ * in all.  The step count of the handle counts the captured call, not its
+ * replays. */
 lbm_status lbm_step(lbm_handle *h, int64_t n);
 
 /* Number of completed steps. */
